@@ -428,29 +428,37 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         M->n_links = iptr[n];
         // incidence records: everything one cache update of Eq. energy_diff_upd
         // needs for a term of at most 4 members, read in one step
-        std::vector<int32_t> inc_rec((size_t)iptr[n] * 12, 0);
+        std::vector<int32_t> inc_rec((size_t)iptr[n] * 16, 0);
         for (int32_t k = 0; k < n; ++k)
             for (int64_t e = iptr[k]; e < iptr[k + 1]; ++e) {
-                int32_t* q = inc_rec.data() + (size_t)e * 12;
+                int32_t* q = inc_rec.data() + (size_t)e * 16;
                 const int32_t tt = inc_term[e];
                 const int32_t nm = term_ptr[tt + 1] - term_ptr[tt];
-                q[0] = tt;
-                q[1] = inc_exp[e];
+                q[7] = tt;
                 if (nm > 4) {
                     q[2] = -1;
                     continue;
                 }
+                if (M->is_float) {
+                    const float c = (float)tcoef_d[tt];
+                    std::memcpy(q, &c, 4);
+                } else {
+                    std::memcpy(q, &tcoef_i[tt], 8);
+                }
                 int c = 0, packed = 0;
+                bool ones = inc_exp[e] == 1;
                 for (int32_t p = term_ptr[tt]; p < term_ptr[tt + 1]; ++p) {
                     const int32_t v = mem_var[p];
                     if (v == k) continue;
                     q[4 + c] = v;
                     packed |= mem_exp[p] << (8 * c);
                     q[8 + c] = slot_of(v, mem_exp[p]);
+                    q[12 + c] = lo[v];
+                    ones = ones && mem_exp[p] == 1;
                     ++c;
                 }
-                q[2] = c;
-                q[7] = packed;
+                q[2] = inc_exp[e] | (c << 8) | (ones ? 1 << 16 : 0);
+                q[3] = packed;
             }
         // neighbours for levels: members of incident interaction terms
         nb_ptr.assign(n + 1, 0);

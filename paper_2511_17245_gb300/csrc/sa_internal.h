@@ -70,11 +70,12 @@ struct DevModel {
     const double* aconst_d;
     const int32_t* inc_term;    // incidence of variable s: interaction terms containing s
     const int32_t* inc_exp;     //   and the exponent of s in that term
-    // per incidence, 12 int32 (three 16-byte groups): {term, exponent of s,
-    // number of other members (0..3, or -1 for terms of more than 4 members),
-    // 0}, {other members' variables v1..v3, their exponents packed
-    // e1 | e2 << 8 | e3 << 16}, {their coefficient slots (slot_base[v] + index
-    // of the exponent), 0}
+    // per incidence, 16 int32 (four 16-byte groups): {coefficient (int64, or
+    // fp32 bits and 0), exponent of s | number of other members (0..3) << 8 |
+    // 1 << 16 when every exponent is 1 (or -1 for terms of more than 4
+    // members), the other members' exponents packed e1 | e2 << 8 | e3 << 16},
+    // {their variables v1..v3, term}, {their coefficient slots (slot_base[v] +
+    // index of the exponent), 0}, {their lower bounds, 0}
     const int32_t* inc_rec;
     const int32_t* term_ptr;    // [n_iterms + 1] into mem_var / mem_exp
     const int32_t* mem_var;     // members (distinct variables) of interaction terms

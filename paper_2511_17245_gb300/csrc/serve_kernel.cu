@@ -16,7 +16,7 @@ namespace dev {
 
 template <class F, class Z, int RULE, int KIND>
 __device__ __noinline__ void serve_body(const SweepArgs& a, int slot, int t, int r, uint8_t* base) {
-    replica_body<F, Z, RULE, KIND>(a, slot, t, r, base);
+    replica_body<F, Z, RULE, KIND, MEM_EITHER>(a, slot, t, r, base);
 }
 
 template <class F, class Z, int KIND>
