@@ -257,7 +257,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
     dm.const_i = (int64_t)const_i;
     dm.const_d = const_d;
     struct Offs {
-        size_t meta, lvl_ptr, lvl_vars, lvl_rec;
+        size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk = 0;
         size_t adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
         size_t slot_base, omega, aconst_i, aconst_f, aconst_d, inc_term, inc_exp, inc_rec, term_ptr, mem_var, mem_exp,
             tcoef_i, tcoef_f, tcoef_d;
@@ -361,6 +361,32 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         off.lvl_vars = blob.add(lvl_vars);
         off.lvl_rec = blob.add(rec);
         off.adj_col = blob.add(col);
+        if (sa::plan_block_model(n, M->n_levels)) {
+            // blocked sweeps: records in index order, the earlier neighbours in
+            // each variable's block of 32 and the block's couplings
+            std::vector<sa::LevelRec> ir(n);
+            for (int32_t L = 0; L < M->n_levels; ++L)
+                for (int32_t i = lvl_ptr[L]; i < lvl_ptr[L + 1]; ++i) {
+                    ir[lvl_vars[i]] = rec[i];
+                    ir[lvl_vars[i]].slot_base = lvl_ptr[L + 1] - lvl_ptr[L];
+                }
+            std::vector<uint32_t> mask(n, 0);
+            const size_t cells = (size_t)((n + 31) / 32) * 32 * 32;
+            std::vector<int64_t> bi(M->is_float ? 0 : cells, 0);
+            std::vector<float> bf(M->is_float ? cells : 0, 0.f);
+            for (int32_t k = 0; k < n; ++k) {
+                const int32_t kb = k / 32 * 32;
+                auto first = std::lower_bound(col.begin() + ptr[k], col.begin() + ptr[k] + deg[k], kb);
+                for (int64_t e = first - col.begin(); e < ptr[k] + deg[k] && col[e] < kb + 32; ++e) {
+                    if (col[e] < k) mask[k] |= 1u << (col[e] - kb);
+                    if (M->is_float) bf[(size_t)k * 32 + (col[e] - kb)] = (float)vd[e];
+                    else bi[(size_t)k * 32 + (col[e] - kb)] = vi[e];
+                }
+            }
+            off.idx_rec = blob.add(ir);
+            off.blk_mask = blob.add(mask);
+            off.blk = M->is_float ? blob.add(bf) : blob.add(bi);
+        }
         if (M->is_float) {
             std::vector<float> vf(vd.size()), lf(n), df(n);
             for (size_t i = 0; i < vd.size(); ++i) vf[i] = (float)vd[i];
@@ -530,6 +556,12 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
     dm.lvl_vars = at<int32_t>(b, off.lvl_vars);
     dm.lvl_rec = at<sa::LevelRec>(b, off.lvl_rec);
     if (dm.kind == sa::KIND_QUIO) {
+        if (sa::plan_block_model(n, M->n_levels)) {
+            dm.idx_rec = at<sa::LevelRec>(b, off.idx_rec);
+            dm.blk_mask = at<uint32_t>(b, off.blk_mask);
+            if (M->is_float) dm.blk_f = at<float>(b, off.blk);
+            else dm.blk_i = at<int64_t>(b, off.blk);
+        }
         dm.adj_col = at<int32_t>(b, off.adj_col);
         if (M->is_float) {
             dm.adj_f = at<float>(b, off.adj_f);
@@ -825,9 +857,10 @@ sa_status sa_run(const sa_model* M, const sa_run_params* p, int32_t* out_states,
     int dev_sms = 0;
     cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev);
     sa::RunPlan plan{};
-    if (const char* err = sa::plan_run_shape(sa::plan_model(view), R, p->threads_per_replica, p->replicas_per_block,
-                                             (p->flags & SA_FLAG_STATE_IN_GLOBAL) != 0, dev_sms,
-                                             sa::sweep_max_shared_optin(), &plan))
+    if (const char* err = sa::plan_run(sa::plan_model(view), p->rule, !(p->flags & SA_FLAG_NO_SPECULATION), R,
+                                       p->threads_per_replica, p->replicas_per_block,
+                                       (p->flags & SA_FLAG_STATE_IN_GLOBAL) != 0, dev_sms,
+                                       sa::sweep_max_shared_optin(), &plan))
         return fail(SA_ERR_INVALID, err);
     const bool in_global = plan.in_global != 0;
     const int rpc = plan.rpc, tpr = plan.tpr, blocks = plan.blocks;
@@ -880,7 +913,6 @@ sa_status sa_run(const sa_model* M, const sa_run_params* p, int32_t* out_states,
     a.key1 = (uint32_t)(p->seed >> 32);
     a.inst = p->instance_id;
     a.refresh_interval = p->refresh_interval > 0 ? p->refresh_interval : 50;
-    a.speculate = (p->flags & SA_FLAG_NO_SPECULATION) ? 0 : 1;
     a.beta = d_tab;
     a.ratio = d_tab + S;
     a.init_states = d_init;
@@ -1042,6 +1074,7 @@ __attribute__((visibility("hidden"))) int sa_internal_model_view(const sa_model*
     v->cache_elems = M->cache_elems;
     v->n_levels = M->n_levels;
     v->max_link_len = M->max_link_len;
+    v->n_links = M->n_links;
     v->de_max = M->de_max;
     v->de_min = M->de_min;
     return 1;

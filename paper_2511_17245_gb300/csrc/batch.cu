@@ -81,6 +81,8 @@ size_t layout(sa::SweepArgs& a, const sa::ModelView& v, int zb, int tpr) {
     sa::RunPlan pl{};
     const int64_t rep = sa::plan_layout(sa::plan_model(v), zb, tpr, &pl);
     pl.rpc = a.rpc;
+    pl.blocked = a.blocked;
+    pl.hb_tpr = a.hb_tpr;
     sa::plan_apply(pl, a);
     return (size_t)rep;
 }
@@ -283,7 +285,7 @@ sa_status sa_batch_create(sa_batch** out, const sa_model* const* models, int32_t
         a.key1 = (uint32_t)(p.seed >> 32);
         a.inst = p.instance_id;
         a.refresh_interval = p.refresh_interval > 0 ? p.refresh_interval : 50;
-        a.speculate = (p.flags & SA_FLAG_NO_SPECULATION) ? 0 : 1;
+        a.blocked = sa::plan_blocked(sa::plan_model(v), p.rule, !(p.flags & SA_FLAG_NO_SPECULATION));
         a.beta = d_tab + tpos;
         a.ratio = d_tab + tpos + S;
         a.init_states = p.init_states;
@@ -305,16 +307,21 @@ sa_status sa_batch_create(sa_batch** out, const sa_model* const* models, int32_t
         delete b;
         return bcuda(e, "copy batch tables");
     }
-    // heuristic shape: threads per replica from the cost-weighted mean level width
-    double wsum = 0, csum = 0;
+    // heuristic shape: threads per replica from the cost-weighted mean of what
+    // the instances can use (half the mean level width, or the threads of a
+    // blocked sweep)
+    double wsum = 0, csum = 0, tsum = 0;
     for (int i = 0; i < n_models; ++i) {
         const sa::ModelView& v = b->views[i];
-        const double c = cost[i] * b->R[i];
-        wsum += c * (double)v.n / (double)std::max(1, v.n_levels);
+        const double c = cost[i] * b->R[i], width = (double)v.n / (double)std::max(1, v.n_levels);
+        wsum += c * width;
+        tsum += c * (b->h_insts[i].blocked ? (double)sa::plan_blocked_threads(sa::plan_model(v)) : width / 2.0);
         csum += c;
     }
-    const double mean_w = wsum / std::max(1.0, csum);
-    int tpr = std::min(256, std::max(32, ((int)std::ceil(mean_w / 2.0) + 31) / 32 * 32));
+    auto whole_warps = [](double x) { return std::min(256, std::max(32, ((int)std::ceil(x) + 31) / 32 * 32)); };
+    const int hb_tpr = whole_warps(wsum / std::max(1.0, csum) / 2.0);
+    for (auto& a : b->h_insts) a.hb_tpr = hb_tpr;
+    const int tpr = whole_warps(tsum / std::max(1.0, csum));
     sa_status st = apply_shape(b, tpr, 0);
     if (st == SA_OK) {
         e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);

@@ -106,9 +106,10 @@ extern "C" sa_status sa_run_noalloc(const sa_model* M, const sa_run_params* p, i
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sa::RunPlan plan{};
-    if (const char* err = sa::plan_run_shape(sa::plan_model(mv), R, p->threads_per_replica, p->replicas_per_block,
-                                             (p->flags & SA_FLAG_STATE_IN_GLOBAL) != 0, sms,
-                                             sa::sweep_max_shared_optin(), &plan))
+    if (const char* err = sa::plan_run(sa::plan_model(mv), p->rule, !(p->flags & SA_FLAG_NO_SPECULATION), R,
+                                       p->threads_per_replica, p->replicas_per_block,
+                                       (p->flags & SA_FLAG_STATE_IN_GLOBAL) != 0, sms,
+                                       sa::sweep_max_shared_optin(), &plan))
         return fail(SA_ERR_INVALID, err);
     const bool in_global = plan.in_global != 0;
     const size_t slab_bytes = in_global ? (size_t)R * (size_t)plan.rep_bytes : 0;
@@ -129,7 +130,6 @@ extern "C" sa_status sa_run_noalloc(const sa_model* M, const sa_run_params* p, i
     a.key1 = (uint32_t)(p->seed >> 32);
     a.inst = p->instance_id;
     a.refresh_interval = p->refresh_interval > 0 ? p->refresh_interval : 50;
-    a.speculate = (p->flags & SA_FLAG_NO_SPECULATION) ? 0 : 1;
     a.beta = d_tab;
     a.ratio = d_tab + S;
     a.init_states = p->init_states;

@@ -46,6 +46,12 @@ struct DevModel {
     const int32_t* lvl_ptr;     // [n_levels + 1]
     const int32_t* lvl_vars;    // [n]: variables grouped by dependency level
     const LevelRec* lvl_rec;    // [n]: their records, same order
+    // models with narrow levels (plan_block_model), swept in blocks of 32
+    // consecutive variables; null otherwise
+    const LevelRec* idx_rec;    // [n]: records in index order, slot_base = width of the variable's level
+    const uint32_t* blk_mask;   // [n]: bit j set iff variable 32 (k / 32) + j < k shares a term with k
+    const int64_t* blk_i;       // [32 ceil(n / 32)][32]: J_kj of the variables j of k's block
+    const float* blk_f;
 
     // QUIO (every term of total degree <= 2):
     //   E = c + sum_k lin_k z_k + sum_k diag_k z_k^2 + sum_{i<j} J_ij z_i z_j
@@ -112,8 +118,8 @@ struct SweepArgs {
     int64_t rep_bytes;          // bytes of one replica's state region
     int32_t off_z, off_cache, off_ctl, off_list, off_red;
     int32_t off_lvl;            // level boundaries staged in the replica region (-1: read from the model)
-    int32_t speculate;          // decide runs of single-variable levels a warp at a time
-    int32_t _pad_spec;
+    int32_t blocked;            // sweep in blocks of 32 variables (the model has idx_rec)
+    int32_t hb_tpr;             // threads per replica that decide the form of heat-bath sums (hb_warp_mode)
     int32_t rpc;                // replicas per block
     int32_t tpr;                // threads per replica (multiple of 32)
     int32_t heavy_links;        // link_len above which updates are cooperative
@@ -212,6 +218,7 @@ struct ModelView {
     int64_t cache_elems;
     int32_t n_levels;
     int32_t max_link_len;       // longest neighbour / incidence list
+    int64_t n_links;
     double de_max, de_min;
 };
 
@@ -244,10 +251,42 @@ struct PlanModel {
     int32_t zbytes;             // bytes of one state offset z_k - l_k
     int32_t max_link_len;
     int64_t cache_elems;        // QUIO: n fields; HUIO: coefficient slots
+    int32_t block_model;        // the model holds the tables of the blocked sweep
+    int32_t dense_rows;         // complete graph
+    int32_t mean_links;         // mean length of the neighbour lists
 };
 
 inline PlanModel plan_model(const ModelView& v) {
-    return PlanModel{v.n, v.n_levels, v.dm.kind, v.is_float, v.zbytes, v.max_link_len, v.cache_elems};
+    return PlanModel{v.n, v.n_levels, v.dm.kind, v.is_float, v.zbytes, v.max_link_len, v.cache_elems,
+                     v.dm.idx_rec != nullptr, v.dm.dense_rows, (int32_t)(v.n_links / (v.n > 0 ? v.n : 1))};
+}
+
+// ------------------------------------------------------------------ blocked sweeps
+// A level costs a group barrier, a Philox block and an L2 round trip whatever
+// its width; a block of 32 variables costs one of each plus a short round per
+// colliding change.  kBlockWidth is the mean level width up to which blocks win
+// (QUIO), kBlockWidthHeat the same for the heat bath, whose decisions a block
+// makes one after the other and a level side by side.
+constexpr int kBlockWidth = 16;
+constexpr int kBlockWidthHeat = 3;
+
+inline bool plan_block_model(int32_t n, int32_t n_levels) { return (int64_t)n <= (int64_t)kBlockWidth * n_levels; }
+
+// Whether a run of this model sweeps in blocks (`allowed`: the caller did not
+// ask for the level order).
+inline bool plan_blocked(const PlanModel& m, int rule, bool allowed) {
+    if (!m.block_model || !allowed) return false;
+    return rule != RULE_HEAT_BATH || (int64_t)m.n <= (int64_t)kBlockWidthHeat * m.n_levels;
+}
+
+// Threads that a replica of a blocked sweep can use: one warp decides; the
+// others add its changes to the other fields (complete graphs: every field,
+// several rows deep; else the rows' links).
+inline int plan_blocked_threads(const PlanModel& m) {
+    if (m.n <= 32) return 32;
+    const int work = m.dense_rows ? m.n / 4 : (4 * m.mean_links < m.n ? 4 * m.mean_links : m.n);
+    const int want = 32 + (work + 31) / 32 * 32;
+    return want > 512 ? 512 : want;
 }
 
 // Per-replica state layout and launch shape of one run.
@@ -261,14 +300,15 @@ struct RunPlan {
     int64_t rep_bytes;          // bytes of one replica's state region
     int64_t shared_bytes;       // dynamic shared memory of one block
     int32_t off_z, off_cache, off_ctl, off_list, off_red, off_lvl;
+    int32_t blocked, hb_tpr;    // see SweepArgs (set by plan_run)
 };
 
 inline int64_t plan_round16(int64_t x) { return (x + 15) / 16 * 16; }
 
 // State layout of one replica for `tpr` threads: offsets z_k - l_k (zbytes
-// each), the cache (int64 or fp32), the control words (three list counters,
-// the flattened length and two 48-byte results of speculative windows), the
-// cooperative update list, the reduction scratch (one 8-byte word
+// each), the cache (int64 or fp32), the control words (three list counters or
+// the commit counts and commands of a blocked sweep), the cooperative update
+// list or a blocked sweep's two commit lists, the reduction scratch (one 8-byte word
 // per warp) and, when it takes at most 16 KB, the level boundary table.
 // `zbytes` may exceed the model's own (a batch uses its widest).  QUIO rows are
 // cheap per entry (one atomic) and go inline up to 64 links; HUIO incidences
@@ -328,6 +368,31 @@ inline const char* plan_run_shape(const PlanModel& m, int32_t R, int32_t tpr_req
     p->in_global = in_global ? 1 : 0;
     p->blocks = (R + rpc - 1) / rpc;
     p->shared_bytes = in_global ? 0 : (int64_t)rpc * rep;
+    return nullptr;
+}
+
+// Plan of a single-model run: plan_run_shape, and for blocked sweeps whose
+// caller left the thread count open, the threads that such a sweep can use
+// within 512 per block.
+inline const char* plan_run(const PlanModel& m, int rule, bool allow_blocks, int32_t R, int32_t tpr_req,
+                            int32_t rpc_req, bool force_global, int sms, int64_t smem_max, RunPlan* p) {
+    if (const char* err = plan_run_shape(m, R, tpr_req, rpc_req, force_global, sms, smem_max, p)) return err;
+    const int32_t hb_tpr = p->tpr;
+    // (the shape does not depend on allow_blocks, so that float energies, summed
+    // in FP64 over the replica's threads, are the same bits either way)
+    const bool blocked = plan_blocked(m, rule, true);
+    if (blocked && tpr_req <= 0) {
+        const int rpc = p->rpc;
+        int tpr = plan_blocked_threads(m);
+        const int cap = 512 / rpc / 32 * 32;
+        tpr = tpr > cap ? cap : tpr;
+        RunPlan q{};
+        // more threads per replica grow its region a little: keep the first plan if that no longer fits
+        if (plan_run_shape(m, R, tpr, rpc, force_global, sms, smem_max, &q) == nullptr && q.in_global == p->in_global)
+            *p = q;
+    }
+    p->blocked = blocked && allow_blocks ? 1 : 0;
+    p->hb_tpr = hb_tpr;
     return nullptr;
 }
 
@@ -399,6 +464,8 @@ inline void plan_apply(const RunPlan& p, SweepArgs& a) {
     a.tpr = p.tpr;
     a.heavy_links = p.heavy_links;
     a.list_cap = p.list_cap;
+    a.blocked = p.blocked;
+    a.hb_tpr = p.hb_tpr;
 }
 
 // Host-side launchers implemented in the .cu files.

@@ -14,9 +14,19 @@
 namespace sa {
 namespace dev {
 
+template <class F, class Z, int RULE, int KIND, bool BLK>
+__device__ __noinline__ void serve_form(const SweepArgs& a, int slot, int t, int r, uint8_t* base) {
+    replica_body<F, Z, RULE, KIND, MEM_EITHER, BLK>(a, slot, t, r, base);
+}
 template <class F, class Z, int RULE, int KIND>
-__device__ __noinline__ void serve_body(const SweepArgs& a, int slot, int t, int r, uint8_t* base) {
-    replica_body<F, Z, RULE, KIND, MEM_EITHER>(a, slot, t, r, base);
+__device__ __forceinline__ void serve_body(const SweepArgs& a, int slot, int t, int r, uint8_t* base) {
+    if constexpr (KIND == KIND_QUIO) {
+        if (a.blocked) {
+            serve_form<F, Z, RULE, KIND, true>(a, slot, t, r, base);
+            return;
+        }
+    }
+    serve_form<F, Z, RULE, KIND, false>(a, slot, t, r, base);
 }
 
 template <class F, class Z, int KIND>

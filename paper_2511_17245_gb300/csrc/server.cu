@@ -175,7 +175,6 @@ bool admit(sa_server* s, Request* r, int slot) {
     a.key1 = (uint32_t)(p.seed >> 32);
     a.inst = p.instance_id;
     a.refresh_interval = p.refresh_interval > 0 ? p.refresh_interval : 50;
-    a.speculate = (p.flags & SA_FLAG_NO_SPECULATION) ? 0 : 1;
     a.beta = reinterpret_cast<const float*>(d + r->o_tab);
     a.ratio = a.beta + S;
     a.out_states = reinterpret_cast<int32_t*>(d + o_st);
@@ -185,6 +184,8 @@ bool admit(sa_server* s, Request* r, int slot) {
     sa::RunPlan pl{};
     sa::plan_layout(sa::plan_model(v), r->zbytes, s->args.tpr, &pl);
     pl.rpc = s->args.rpc;
+    pl.blocked = sa::plan_blocked(sa::plan_model(v), p.rule, !(p.flags & SA_FLAG_NO_SPECULATION));
+    pl.hb_tpr = s->args.tpr;
     sa::plan_apply(pl, a);
     sa::ServeReq& q = s->h_reqs[slot];
     q.args = a;

@@ -137,6 +137,8 @@ struct Coef;
 template <>
 struct Coef<long long> {
     __device__ static long long adj(const DevModel& m, int i) { return m.adj_i[i]; }
+    __device__ static long long adj_once(const DevModel& m, int i) { return __ldcg((const long long*)m.adj_i + i); }
+    __device__ static const long long* blk(const DevModel& m) { return (const long long*)m.blk_i; }
     __device__ static long long lin(const DevModel& m, int k) { return m.lin_i[k]; }
     __device__ static long long diag(const DevModel& m, int k) { return m.diag_i[k]; }
     __device__ static long long aconst(const DevModel& m, int s) { return m.aconst_i[s]; }
@@ -145,6 +147,8 @@ struct Coef<long long> {
 template <>
 struct Coef<float> {
     __device__ static float adj(const DevModel& m, int i) { return __ldg(m.adj_f + i); }
+    __device__ static float adj_once(const DevModel& m, int i) { return __ldcg(m.adj_f + i); }
+    __device__ static const float* blk(const DevModel& m) { return m.blk_f; }
     __device__ static float lin(const DevModel& m, int k) { return __ldg(m.lin_f + k); }
     __device__ static float diag(const DevModel& m, int k) { return __ldg(m.diag_f + k); }
     __device__ static float aconst(const DevModel& m, int s) { return __ldg(m.aconst_f + s); }
@@ -664,8 +668,13 @@ __device__ __forceinline__ float quio_w(float dz, float A, float B, float C) {
 // fast approximate divide, reciprocal square root and logarithm (relative
 // errors of a few ulp); the weights themselves are computed as elsewhere.
 // `temp` is T = 1 / beta.
-__device__ __forceinline__ long long heat_bath_quio_f32_small(float f, float d, long long z, long long lo,
-                                                              uint32_t width, uint32_t xu, float beta, float temp) {
+struct HbWindow {
+    int n, base, nrb;            // values of the range, first value of the window, its blocks of 16
+    float dz0, dzb0;             // v - z at the first value of the range / of the window
+    float hA, hB, mb;            // weight coefficients (quio_w)
+};
+__device__ __forceinline__ HbWindow hb_small_window(float f, float d, long long z, long long lo, uint32_t width,
+                                                    float beta, float temp) {
     const int n = (int)width + 1;
     const float zf = __int2float_rn((int)z);
     const float dz0 = __int2float_rn((int)(lo - z));
@@ -698,7 +707,14 @@ __device__ __forceinline__ long long heat_bath_quio_f32_small(float f, float d, 
     const int kb0 = (int)(wlo - dz0) >> 4, kb1 = (int)(whi - dz0) >> 4;
     const int base = kb0 * 16;
     const int nrb = kb1 - kb0 + 1;
-    const float dzb0 = dz0 + (float)base;
+    return {n, base, nrb, dz0, dz0 + (float)base, hA, hB, mb};
+}
+
+__device__ __forceinline__ long long heat_bath_quio_f32_small(float f, float d, long long z, long long lo,
+                                                              uint32_t width, uint32_t xu, float beta, float temp) {
+    const HbWindow q = hb_small_window(f, d, z, lo, width, beta, temp);
+    const int n = q.n, base = q.base, nrb = q.nrb;
+    const float dz0 = q.dz0, dzb0 = q.dzb0, hA = q.hA, hB = q.hB, mb = q.mb;
     // block sums in registers (the loops are unrolled, so bs[] is indexed by
     // constants); both loops stop after the window's nrb blocks
     float bs[16];
@@ -1150,6 +1166,48 @@ __device__ __noinline__ void keep_best(const SweepArgs& a, const Z* zs, int r, i
     named_bar(bar_id, tpr);   // every thread has read zs before the next sweep changes it
 }
 
+// ------------------------------------------------------------------ end of a sweep
+// FP64 refresh of float fields and energy when it is due, the per-sweep energy
+// trace and the best state.  `first`: sweep s is the run's first.
+template <class F, class Z, int KIND>
+__device__ __forceinline__ void end_of_sweep(const SweepArgs& a, const Z* zs, F* cache, typename Num<F>::Acc* red,
+                                             int t, int tpr, int bar_id, int r, int s, bool first,
+                                             typename Num<F>::Acc& eacc, float& dacc, float& drift) {
+    using Acc = typename Num<F>::Acc;
+    const DevModel& m = a.m;
+    if constexpr (Num<F>::is_float) {
+        eacc += (double)dacc;
+        dacc = 0.f;
+        const bool last = (s + 1 == a.S);
+        if (last || (a.refresh_interval > 0 && (s + 1) % a.refresh_interval == 0)) {
+            Acc f1 = 0, f2 = 0;
+            if constexpr (KIND == KIND_QUIO) {
+                quio_recompute<F, Z>(m, zs, cache, t, tpr, true, drift, f1, f2);
+                Acc pair2 = group_sum<Acc>(f2, red, t, tpr, bar_id);
+                eacc = f1 + (t == 0 ? pair2 / 2 : Acc(0));
+            } else {
+                huio_recompute<F, Z>(m, zs, cache, t, tpr, true, drift, f1, f2);
+                eacc = f1 + f2;
+                named_bar(bar_id, tpr);
+            }
+            if (t == 0) eacc += m.const_d;
+        }
+    }
+    if (a.energy_trace != nullptr || a.best_states != nullptr) {
+        const Acc tot = group_sum<Acc>(eacc, red, t, tpr, bar_id);   // the same in every thread
+        if (a.energy_trace != nullptr && t == 0) reinterpret_cast<Acc*>(a.energy_trace)[(size_t)s * a.R + r] = tot;
+        if (a.best_states != nullptr) keep_best<Acc, Z>(a, zs, r, t, tpr, bar_id, tot, first);
+    }
+}
+
+}  // namespace dev
+}  // namespace sa
+
+#include "sweep_block.cuh"
+
+namespace sa {
+namespace dev {
+
 // ------------------------------------------------------------------ one replica
 // Sweeps [s0, s1) of the SA run of replica r (Sect. 3.1) by the `tpr` threads
 // of one group; `base` is the group's state region (shared or global memory).
@@ -1159,7 +1217,10 @@ __device__ __noinline__ void keep_best(const SweepArgs& a, const Z* zs, int r, i
 // s1 = S writes the outputs; otherwise it saves its state at `save` (layout:
 // bytes [0, off_ctl) of the state region, then per thread the energy
 // accumulator, the change count and the refresh drift, 24 bytes each).
-template <class F, class Z, int RULE, int KIND, int MEM>
+// BLK: the sweeps go in blocks of variables (sweep_block.cuh) instead of levels.
+// The two are separate instantiations: in one kernel the registers that either
+// keeps across a call of the other were spilled in the level loop.
+template <class F, class Z, int RULE, int KIND, int MEM, bool BLK>
 __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot, const int t, const int r,
                                              uint8_t* base, const int s0 = 0, int s1 = -1,
                                              const uint8_t* restore = nullptr, uint8_t* save = nullptr) {
@@ -1170,7 +1231,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
     if (s1 < 0) s1 = a.S;
     Z* zs = reinterpret_cast<Z*>(base + a.off_z);
     F* cache = reinterpret_cast<F*>(base + a.off_cache);
-    // [0..2] list counters, [3] flattened length, [4..27] two results of speculative windows
+    // [0..2] list counters; blocked sweeps: [0..1] commits of the two lists, [4..7] commands
     int* ctl = reinterpret_cast<int*>(base + a.off_ctl);
     // [cap][6]: variable k, z_old, z_new, link_begin, link_len, prefix of the
     // flattened (entry, link) pairs
@@ -1334,8 +1395,14 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
         const int b0 = lvl_at(L), b1 = lvl_at(L + 1);
         for (int i = b0 + t; i < b1; i += tpr) prefetch_l1(m.lvl_rec + i);
     };
+    if constexpr (BLK) {
+        SweepAcc<F> io{eacc, changes, 0.f, drift, 0, -1};
+        block_run<F, Z, RULE, MEM>(a, base, bar_id, t, r, s0, s1, restore == nullptr, io);
+        eacc = io.e;
+        changes = io.changes;
+        drift = io.drift;
+    } else {
     prefetch_level(0);
-    int win = 0;   // speculative windows run so far (their result slots alternate)
     for (int s = s0; s < s1; ++s) {
         const float beta = __ldg(a.beta + s);
         const float temp = 1.f / beta;
@@ -1347,105 +1414,8 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
             // heat bath over wide ranges gives a narrow level's variables a warp each
             bool wmode = false;
             if constexpr (RULE == RULE_HEAT_BATH)
-                wmode = hb_warp_mode(le - lb, tpr, m.max_width,
+                wmode = hb_warp_mode(le - lb, a.hb_tpr, m.max_width,
                                      Num<F>::is_float && KIND == KIND_QUIO && m.max_width < 256u);
-            // (QUIO only, and neither float heat bath nor heat bath in warp mode:
-            // second inlined copies of their decision or update code would make
-            // the kernel spill registers)
-            constexpr bool kSpeculative = KIND == KIND_QUIO && !(RULE == RULE_HEAT_BATH && Num<F>::is_float);
-            if constexpr (kSpeculative) if (a.speculate && le - lb == 1 && !wmode) {
-                // ---- a run of single-variable levels (every level of a complete
-                // graph), decided by the lanes of warp 0, up to 32 levels at a
-                // time, lane i deciding level L + i.  Every decision before the first one that changes
-                // its variable saw the state of the level-by-level order, since
-                // nothing changed before it, and so did that one; the group then
-                // updates that variable's neighbours and the next window starts
-                // after it.  Results equal those of the level-by-level order; the
-                // energy change and the count go to thread 0 as they do there.
-                int* res = ctl + 4 + 12 * (win & 1);   // {k or -1, levels done, row begin, row length,
-                                                      //  z_old (2), z_new (2), dE (2)}
-                if (t < 32) {
-                    const int lane = t;
-                    const int Li = L + lane;
-                    int idx = 0;
-                    bool single = false;
-                    if (Li < m.n_levels) {
-                        idx = lvl_at(Li);
-                        single = lvl_at(Li + 1) - idx == 1;
-                    }
-                    const unsigned multi = __ballot_sync(0xffffffffu, !single);
-                    const int w = multi ? __ffs(multi) - 1 : 32;   // >= 1: level L holds one variable
-                    long long zz = 0, vv2 = 0;
-                    F d2 = F(0);
-                    LevelRec rc{};
-                    int p = w;           // levels decided without a change
-                    bool chg = false;    // level L + p changed its variable
-                    if (lane < w) {
-                        rc = load_rec(idx);
-                        decide(rc, s, beta, temp, ratio, zz, vv2, d2, false);
-                    }
-                    {
-                        const unsigned c = __ballot_sync(0xffffffffu, lane < w && vv2 != zz);
-                        if (c) {
-                            p = __ffs(c) - 1;
-                            chg = true;
-                        }
-                        if (a.trace != nullptr && r < a.trace_R && (lane < p || (chg && lane == p)))
-                            a.trace[((size_t)s * a.trace_R + r) * m.n + rc.k] = (int32_t)vv2;
-                        // the changing lane's decision goes to lane 0
-                        if (chg) {
-                            const int k2 = __shfl_sync(0xffffffffu, rc.k, p);
-                            const int lo2 = __shfl_sync(0xffffffffu, rc.lo, p);
-                            const int b2 = __shfl_sync(0xffffffffu, rc.link_begin, p);
-                            const int l2 = __shfl_sync(0xffffffffu, rc.link_len, p);
-                            zz = __shfl_sync(0xffffffffu, zz, p);
-                            vv2 = __shfl_sync(0xffffffffu, vv2, p);
-                            d2 = __shfl_sync(0xffffffffu, d2, p);
-                            rc.k = k2;
-                            rc.lo = lo2;
-                            rc.link_begin = b2;
-                            rc.link_len = l2;
-                        }
-                    }
-                    if (lane == 0) {
-                        res[0] = chg ? rc.k : -1;
-                        res[1] = chg ? p + 1 : w;
-                        if (chg) {
-                            zs[rc.k] = (Z)(vv2 - (long long)rc.lo);
-                            res[2] = rc.link_begin;
-                            res[3] = rc.link_len;
-                            *reinterpret_cast<long long*>(res + 4) = zz;
-                            *reinterpret_cast<long long*>(res + 6) = vv2;
-                            *reinterpret_cast<F*>(res + 8) = d2;
-                        }
-                    }
-                }
-                named_bar(bar_id, tpr);
-                const int kk = res[0];
-                if (kk >= 0) {
-                    const int rb = res[2], rl = res[3];
-                    const long long zold = *reinterpret_cast<const long long*>(res + 4);
-                    const long long znew = *reinterpret_cast<const long long*>(res + 6);
-                    if (t == 0) {
-                        if constexpr (Num<F>::is_float) dacc += (float)*reinterpret_cast<const F*>(res + 8);
-                        else eacc += (Acc)*reinterpret_cast<const F*>(res + 8);
-                        ++changes;
-                    }
-                    if (m.dense_rows) {
-                        // row kk lists every j != kk in order: its columns need no reads
-                        for (int e = t; e < rl; e += tpr)
-                            solo_add(cache + e + (e >= kk ? 1 : 0), Coef<F>::adj(m, rb + e), znew - zold);
-                    } else {
-                        for (int e = rb + t; e < rb + rl; e += tpr)
-                            solo_add(cache + __ldg(m.adj_col + e), Coef<F>::adj(m, e), znew - zold);
-                    }
-                    named_bar(bar_id, tpr);
-                }
-                L += res[1] - 1;
-                ++win;
-                gl3 = gl3 == 2 ? 0 : gl3 + 1;
-                continue;
-            }
             // the next level (the first level of the next sweep after the last)
             if (L + 1 < m.n_levels) prefetch_level(L + 1);
             else if (s + 1 < a.S) prefetch_level(0);
@@ -1587,31 +1557,9 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
             }
             gl3 = gl3 == 2 ? 0 : gl3 + 1;
         }
-        // ---- FP64 refresh of float fields and energy
-        if constexpr (Num<F>::is_float) {
-            eacc += (double)dacc;
-            dacc = 0.f;
-            const bool last = (s + 1 == a.S);
-            if (last || (a.refresh_interval > 0 && (s + 1) % a.refresh_interval == 0)) {
-                Acc f1 = 0, f2 = 0;
-                if constexpr (KIND == KIND_QUIO) {
-                    quio_recompute<F, Z>(m, zs, cache, t, tpr, true, drift, f1, f2);
-                    Acc pair2 = group_sum<Acc>(f2, red, t, tpr, bar_id);
-                    eacc = f1 + (t == 0 ? pair2 / 2 : Acc(0));
-                } else {
-                    huio_recompute<F, Z>(m, zs, cache, t, tpr, true, drift, f1, f2);
-                    eacc = f1 + f2;
-                    named_bar(bar_id, tpr);
-                }
-                if (t == 0) eacc += m.const_d;
-            }
-        }
-        if (a.energy_trace != nullptr || a.best_states != nullptr) {
-            const Acc tot = group_sum<Acc>(eacc, red, t, tpr, bar_id);   // the same in every thread
-            if (a.energy_trace != nullptr && t == 0) reinterpret_cast<Acc*>(a.energy_trace)[(size_t)s * a.R + r] = tot;
-            if (a.best_states != nullptr)
-                keep_best<Acc, Z>(a, zs, r, t, tpr, bar_id, tot, s == s0 && restore == nullptr);
-        }
+        end_of_sweep<F, Z, KIND>(a, zs, cache, red, t, tpr, bar_id, r, s, s == s0 && restore == nullptr, eacc, dacc,
+                                 drift);
+    }
     }
 
     if (save != nullptr) {
@@ -1649,7 +1597,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
 
 // ------------------------------------------------------------------ kernels
 // One instance: replica blockIdx.x * rpc + slot per thread group.
-template <class F, class Z, int RULE, int KIND, bool SMEM>
+template <class F, class Z, int RULE, int KIND, bool SMEM, bool BLK>
 __global__ void __launch_bounds__(512, 1) sweep_kernel(const SweepArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     const int slot = threadIdx.x / a.tpr;
@@ -1657,7 +1605,7 @@ __global__ void __launch_bounds__(512, 1) sweep_kernel(const SweepArgs a) {
     const int r = blockIdx.x * a.rpc + slot;
     if (slot >= a.rpc || r >= a.R) return;
     uint8_t* base = SMEM ? (smem_raw + (size_t)slot * (size_t)a.rep_bytes) : (a.gstate + (size_t)r * (size_t)a.rep_bytes);
-    replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL>(a, slot, t, r, base);
+    replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL, BLK>(a, slot, t, r, base);
 }
 
 __device__ __forceinline__ unsigned int ld_acquire_gpu(const unsigned int* p) {
@@ -1681,7 +1629,7 @@ constexpr unsigned long long kHandoffSpinLimit = 1ull << 32;
 // it, runs its sweeps and saves the state for the next chunk.  Per-replica
 // results equal those of sweep_kernel: every chunk draws the same Philox
 // counters and the saved state includes the per-thread accumulators.
-template <class F, class Z, int RULE, int KIND>
+template <class F, class Z, int RULE, int KIND, bool BLK>
 __global__ void __launch_bounds__(512, 1) sweep_sliced_kernel(const SweepArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     __shared__ int task_s[16][2];
@@ -1725,7 +1673,7 @@ __global__ void __launch_bounds__(512, 1) sweep_sliced_kernel(const SweepArgs a)
         const int32_t s0 = j * K, s1 = min(a.S, s0 + K);
         uint8_t* region = a.handoff + (size_t)r * (size_t)a.handoff_bytes;
         if (j > 0) __threadfence();
-        replica_body<F, Z, RULE, KIND, MEM_SHARED>(a, slot, t, r, base, s0, s1, j > 0 ? region : nullptr,
+        replica_body<F, Z, RULE, KIND, MEM_SHARED, BLK>(a, slot, t, r, base, s0, s1, j > 0 ? region : nullptr,
                                        s1 < a.S ? region : nullptr);
         if (s1 < a.S) {
             __threadfence();
@@ -1733,6 +1681,16 @@ __global__ void __launch_bounds__(512, 1) sweep_sliced_kernel(const SweepArgs a)
             if (t == 0) st_release_gpu(a.handoff_flag + r, (unsigned int)(j + 1));
         }
     }
+}
+
+// One unit of a batch, out of line where instances of both sweep forms share a
+// kernel.  The shared-memory base is formed here, so that its address space
+// stays known.
+template <class F, class Z, int RULE, int KIND, bool SMEM, bool BLK>
+__device__ __noinline__ void batch_body(const SweepArgs& a, int slot, int t, int r, int64_t slot_bytes, uint8_t* base) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    if (SMEM) base = smem_raw + (size_t)slot * (size_t)slot_bytes;
+    replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL, BLK>(a, slot, t, r, base);
 }
 
 // Many instances in one persistent launch: every thread group repeatedly claims
@@ -1760,7 +1718,15 @@ __global__ void __launch_bounds__(512, 1) batch_kernel(const BatchArgs b) {
         uint32_t* dst = reinterpret_cast<uint32_t*>(&args_s[slot]);
         for (int w = t; w < (int)(sizeof(SweepArgs) / 4); w += b.tpr) dst[w] = src[w];
         named_bar(bar_id, b.tpr);
-        replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL>(args_s[slot], slot, t, un.replica, base);
+        if constexpr (KIND == KIND_QUIO) {
+            if (args_s[slot].blocked)
+                batch_body<F, Z, RULE, KIND, SMEM, true>(args_s[slot], slot, t, un.replica, b.slot_bytes, base);
+            else
+                batch_body<F, Z, RULE, KIND, SMEM, false>(args_s[slot], slot, t, un.replica, b.slot_bytes, base);
+        } else {
+            replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL, false>(args_s[slot], slot, t, un.replica,
+                                                                                   base);
+        }
         named_bar(bar_id, b.tpr);   // the group is done with args_s and unit_s
     }
 }

@@ -6,15 +6,22 @@
 
 namespace sa {
 
-template <class F, class Z, int RULE, int KIND, bool SMEM>
-static int launch_one(const SweepArgs& a, int blocks, int threads, size_t shared_bytes, cudaStream_t st) {
-    auto kern = dev::sweep_kernel<F, Z, RULE, KIND, SMEM>;
+template <class F, class Z, int RULE, int KIND, bool SMEM, bool BLK>
+static int launch_form(const SweepArgs& a, int blocks, int threads, size_t shared_bytes, cudaStream_t st) {
+    auto kern = dev::sweep_kernel<F, Z, RULE, KIND, SMEM, BLK>;
     if (shared_bytes > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_bytes);
         if (e != cudaSuccess) return (int)e;
     }
     kern<<<blocks, threads, shared_bytes, st>>>(a);
     return (int)cudaGetLastError();
+}
+
+template <class F, class Z, int RULE, int KIND, bool SMEM>
+static int launch_one(const SweepArgs& a, int blocks, int threads, size_t sh, cudaStream_t st) {
+    if constexpr (KIND == KIND_QUIO)
+        if (a.blocked) return launch_form<F, Z, RULE, KIND, SMEM, true>(a, blocks, threads, sh, st);
+    return launch_form<F, Z, RULE, KIND, SMEM, false>(a, blocks, threads, sh, st);
 }
 
 template <class F, class Z, int KIND, bool SMEM>
@@ -39,10 +46,10 @@ static int launch_family(const SweepArgs& a, int zbytes, int rule, bool smem, in
     return launch_rule<F, uint32_t, KIND, false>(a, rule, blocks, threads, sh, st);
 }
 
-template <class F, class Z, int RULE, int KIND>
-static int launch_sliced_one(const SweepArgs& a, int grid, int threads, size_t shared_bytes, cudaStream_t st,
-                             int* blocks_per_sm) {
-    auto kern = dev::sweep_sliced_kernel<F, Z, RULE, KIND>;
+template <class F, class Z, int RULE, int KIND, bool BLK>
+static int launch_sliced_form(const SweepArgs& a, int grid, int threads, size_t shared_bytes, cudaStream_t st,
+                              int* blocks_per_sm) {
+    auto kern = dev::sweep_sliced_kernel<F, Z, RULE, KIND, BLK>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_bytes);
     if (e != cudaSuccess) return (int)e;
     if (grid == 0) {
@@ -53,6 +60,13 @@ static int launch_sliced_one(const SweepArgs& a, int grid, int threads, size_t s
     void* params[] = {&args};
     e = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(threads), params, shared_bytes, st);
     return (int)e;
+}
+
+template <class F, class Z, int RULE, int KIND>
+static int launch_sliced_one(const SweepArgs& a, int grid, int threads, size_t sh, cudaStream_t st, int* bps) {
+    if constexpr (KIND == KIND_QUIO)
+        if (a.blocked) return launch_sliced_form<F, Z, RULE, KIND, true>(a, grid, threads, sh, st, bps);
+    return launch_sliced_form<F, Z, RULE, KIND, false>(a, grid, threads, sh, st, bps);
 }
 
 template <class F, class Z, int KIND>
