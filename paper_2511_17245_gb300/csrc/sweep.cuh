@@ -126,6 +126,11 @@ __device__ __forceinline__ void atomic_add_field(long long* p, long long v) {
 
 // Floor division for int64 with positive divisor.
 __device__ __forceinline__ long long floor_div(long long a, long long b) {
+    if (a == (long long)(int)a && b == (long long)(int)b) {   // a fraction of the 64-bit division's cost
+        const int x = (int)a, y = (int)b;
+        const int q = x / y;
+        return q - (x % y != 0 && x < 0 ? 1 : 0);
+    }
     long long q = a / b;
     if ((a % b != 0) && (a < 0)) --q;
     return q;
@@ -524,6 +529,48 @@ __device__ long long heat_bath_general(const VarView<F, KIND>& vv, long long z, 
     }
 }
 
+// heat_bath_general of an integer QUIO variable with at most 32 values, one
+// lane, bit for bit the same pick: the one block of values is always kept, dE
+// walks up by exact differences, and the running sums of the first pass, which
+// the second pass would form again, stay in registers.  Sixteen values take
+// about a quarter of the time of the three loops.
+__device__ __forceinline__ long long heat_bath_narrow(const VarView<long long, KIND_QUIO>& vv, long long z,
+                                                      long long lo, uint32_t width, uint32_t xu, float beta,
+                                                      uint32_t max_width) {
+    long long mn = quio_interval_min<long long>(vv, z, lo, lo + (long long)width);
+    mn = mn < 0 ? mn : 0;
+    long long de = vv.delta(z, lo) - mn;
+    long long step = vv.f + vv.d * (2 * lo + 1);   // dE(v + 1) - dE(v) at v = lo
+    float run[32];
+    float sum = 0.f, comp = 0.f;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) run[8 * g + j] = 0.f;
+        if (8u * g <= max_width) {   // the same for every lane
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if ((uint32_t)(8 * g + j) <= width) {
+                    const float w = expf(-(Num<long long>::to_f(de) * beta));
+                    const float y = w - comp;
+                    const float t = sum + y;
+                    comp = (t - sum) - y;
+                    sum = t;
+                    run[8 * g + j] = sum;
+                }
+                de += step;
+                step += 2 * vv.d;
+            }
+        }
+    }
+    const float thr = unit_open_left(xu) * sum;
+    int pick = (int)width;
+#pragma unroll
+    for (int i = 31; i >= 0; --i)
+        if (run[i] >= thr) pick = i;   // (thr > 0: a value past the range holds 0)
+    return lo + (long long)pick;
+}
+
 // ------------------------------------------------------------------ warp-parallel heat bath
 // A pair hi + lo added with Knuth's TwoSum: the rounding error of hi + hi' is
 // kept in lo, so that sums over many lanes stay within a few ulp.
@@ -826,6 +873,35 @@ __device__ __forceinline__ long long heat_bath_linear(float a, long long lo, uin
 template <class F, class Z>
 __device__ void quio_recompute(const DevModel& m, const Z* zs, F* cache, int t, int tpr, bool measure,
                                float& drift, typename Num<F>::Acc& e_ld, typename Num<F>::Acc& e_pair2) {
+    if constexpr (Num<F>::is_float) {
+        if (m.dense_rows && m.adj_d == nullptr) {
+            // complete graph: thread k takes J_jk from row j (J is symmetric), so
+            // that neighbouring threads read neighbouring entries; row k itself,
+            // walked by one thread, is one sector per entry.  The terms are added
+            // in the same order (j ascending), two fields per thread at a time.
+            for (int k0 = t; k0 < m.n; k0 += 2 * tpr) {
+                const int k1 = k0 + tpr < m.n ? k0 + tpr : k0;
+                double f0 = m.lin_d[k0], f1 = m.lin_d[k1];
+#pragma unroll 4
+                for (int j = 0; j < m.n; ++j) {
+                    const VarMeta mj = m.meta[j];
+                    const double zj = __int2double_rn(mj.lo + (int)zs[j]);
+                    if (j != k0) f0 += (double)__ldcg(m.adj_f + mj.link_begin + k0 - (k0 > j ? 1 : 0)) * zj;
+                    if (j != k1) f1 += (double)__ldcg(m.adj_f + mj.link_begin + k1 - (k1 > j ? 1 : 0)) * zj;
+                }
+                auto put = [&](int k, double f) {
+                    const double zk = __int2double_rn(m.meta[k].lo + (int)zs[k]);
+                    if (measure) drift = fmaxf(drift, (float)fabs((double)cache[k] - f));
+                    cache[k] = (float)f;
+                    e_ld += zk * (m.lin_d[k] + m.diag_d[k] * zk);
+                    e_pair2 += zk * (f - m.lin_d[k]);
+                };
+                put(k0, f0);
+                if (k1 != k0) put(k1, f1);
+            }
+            return;
+        }
+    }
     for (int k = t; k < m.n; k += tpr) {
         const VarMeta mt = m.meta[k];
         const long long zk = (long long)mt.lo + (long long)zs[k];
@@ -1328,6 +1404,12 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
                         done = true;
                     }
                 }
+                if constexpr (!Num<F>::is_float && KIND == KIND_QUIO) {
+                    if (m.max_width < 32u) {
+                        v = heat_bath_narrow(vv, z, lo, rc.width, x.x0, beta, m.max_width);
+                        done = true;
+                    }
+                }
                 if (!done) v = heat_bath_general<F, KIND>(vv, z, lo, rc.width, x.x0, beta);
             }
             if (v != z) de = vv.delta(z, v);
@@ -1396,7 +1478,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
         for (int i = b0 + t; i < b1; i += tpr) prefetch_l1(m.lvl_rec + i);
     };
     if constexpr (BLK) {
-        SweepAcc<F> io{eacc, changes, 0.f, drift, 0, -1};
+        SweepAcc<F> io{eacc, changes, 0.f, drift, 0, 0, -1};
         block_run<F, Z, RULE, MEM>(a, base, bar_id, t, r, s0, s1, restore == nullptr, io);
         eacc = io.e;
         changes = io.changes;

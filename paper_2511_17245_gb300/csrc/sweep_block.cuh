@@ -29,9 +29,16 @@ struct SweepAcc {
     unsigned long long changes;
     float de;                        // float models: energy changes since the last fold into e
     float drift;                     // float models: largest error of a field seen by a refresh
+    int busy;                        // heat bath: changes of the last block
     int par;                         // blocked sweeps: which of the two commit lists is current
     int last;                        // and the block whose changes are not applied everywhere yet (-1: none)
 };
+
+// Heat bath over narrow ranges: a round of lane decisions settles 1 / p
+// variables when a share p of them changes and costs about 750 cycles (16
+// values), deciding them in turn about 550 each; above this many changes in the
+// last block they go in turn (the results are the same).
+constexpr int kBusyBlock = 22;
 
 // A change of the block: {variable, z_new - z_old, first entry and length of its row}.
 using Commit = int4;
@@ -144,36 +151,95 @@ __device__ __forceinline__ long long heat_bath_small_warp(float f, float d, long
     return lo + (long long)(first + (h2 ? __ffs(h2) - 1 : cnt - 1));
 }
 
-// ------------------------------------------------------------------ changes to the other fields
-// Field j of a complete graph: the commits' couplings to it, in order.  Row k
-// lists every j != k in order, so entry j - [j > k] of the row is J_kj.  Rows
-// are read past L1 (each entry is used once) and eight at a time.
+// One variable's heat-bath draw by a whole warp (out of line: four forms that
+// would each hold registers of the block loop).
 template <class F>
-__device__ __forceinline__ F add_commits(const DevModel& m, F f, const Commit* list, int count, int j) {
-    for (int c = 0; c < count; c += 8) {
-        F w[8];
-        int dz[8];
+__device__ __noinline__ int heat_bath_in_turn(F f, F d, int z, int lo, uint32_t width, uint32_t xu, float beta,
+                                              float temp, int lane, bool wide) {
+    VarView<F, KIND_QUIO> vv;
+    vv.f = f;
+    vv.d = d;
+    if (vv.linear()) return (int)heat_bath_linear(Num<F>::to_f(f), lo, width, xu, beta);
+    if (wide) return (int)heat_bath_warp<F, KIND_QUIO>(vv, z, lo, width, xu, beta, lane);
+    if (Num<F>::is_float && width < 256u && lo > -(1 << 22) && (long long)lo + (long long)width < (1 << 22))
+        return (int)heat_bath_small_warp((float)f, (float)d, z, lo, width, xu, beta, temp, lane);
+    if (width < kChainValues) return (int)heat_bath_chain<F>(vv, z, lo, width, xu, beta, lane);
+    return (int)heat_bath_general<F, KIND_QUIO>(vv, z, lo, width, xu, beta);
+}
+
+// ------------------------------------------------------------------ changes to the other fields
+// A pointer into shared memory whose address space the compiler can see (for
+// functions out of line, which are given generic pointers).
+template <int MEM, class T>
+__device__ __forceinline__ T* in_shared(T* p) {
+    if constexpr (MEM == MEM_SHARED) return static_cast<T*>(__cvta_shared_to_generic(__cvta_generic_to_shared(p)));
+    else return p;
+}
+
+// Fields of a complete graph: the commits' couplings to field j, in order.  Row
+// k lists every j != k in order, so entry j - [j > k] of the row is J_kj.  Rows
+// are read past L1 (each entry is used once), kRows at a time and for NF fields
+// at a time, all loads before the first addition.
+template <class F>
+constexpr int kRows = Num<F>::is_float ? 8 : 4;
+template <class F, int NF>
+struct RowPart {
+    F w[NF][kRows<F>];
+};
+template <class F, int NF>
+__device__ __forceinline__ void load_rows(RowPart<F, NF>& q, const DevModel& m, const Commit* list, int c, int count,
+                                          const int (&j)[NF]) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            dz[u] = 0;
-            if (c + u < count) {
-                const Commit e = list[c + u];
-                dz[u] = e.y;
-                w[u] = Coef<F>::adj_once(m, e.z + j - (j > e.x ? 1 : 0));
-            }
+    for (int u = 0; u < kRows<F>; ++u)
+        if (c + u < count) {
+            const Commit e = list[c + u];
+#pragma unroll
+            for (int i = 0; i < NF; ++i)
+                if (j[i] >= 0) q.w[i][u] = Coef<F>::adj_once(m, e.z + j[i] - (j[i] > e.x ? 1 : 0));
+        }
+}
+template <class F, int NF>
+__device__ __forceinline__ void add_rows(const RowPart<F, NF>& q, const Commit* list, int c, int count, F (&f)[NF]) {
+#pragma unroll
+    for (int u = 0; u < kRows<F>; ++u)
+        if (c + u < count) {
+            const int dz = list[c + u].y;
+#pragma unroll
+            for (int i = 0; i < NF; ++i) solo_add(&f[i], q.w[i][u], dz);
+        }
+}
+// Every field outside of blocks b0 and b1, by threads t = 0..nt-1.
+template <class F, int MEM>
+__device__ __noinline__ void add_commits(const DevModel& m, F* cache_any, const Commit* list_any, int count, int b0,
+                                         int b1, int t, int nt) {
+    F* cache = in_shared<MEM>(cache_any);
+    const Commit* list = in_shared<MEM>(list_any);
+    for (int j0 = t; j0 < m.n; j0 += 2 * nt) {
+        int j[2] = {j0, j0 + nt};
+        if ((j[0] >> 5) == b0 || (j[0] >> 5) == b1) j[0] = -1;
+        if (j[1] >= m.n || (j[1] >> 5) == b0 || (j[1] >> 5) == b1) j[1] = -1;
+        F f[2] = {F(0), F(0)};
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (j[i] >= 0) f[i] = cache[j[i]];
+        for (int c = 0; c < count; c += kRows<F>) {
+            RowPart<F, 2> q;
+            load_rows<F, 2>(q, m, list, c, count, j);
+            add_rows<F, 2>(q, list, c, count, f);
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (c + u < count) solo_add(&f, w[u], dz[u]);
+        for (int i = 0; i < 2; ++i)
+            if (j[i] >= 0) cache[j[i]] = f[i];
     }
-    return f;
 }
 
 // The commits' rows by columns, any graph: every thread of `nt` takes the next
 // (commit, link) pair.  Columns of block `own` already have the change.
 template <class F, int MEM>
-__device__ __forceinline__ void scatter_commits(const DevModel& m, F* cache, const Commit* list, int count, int own,
-                                                int t, int nt) {
+__device__ __noinline__ void scatter_commits(const DevModel& m, F* cache_any, const Commit* list_any, int count, int own,
+                                             int t, int nt) {
+    F* cache = in_shared<MEM>(cache_any);
+    const Commit* list = in_shared<MEM>(list_any);
     const int lane = t & 31;
     const int len = lane < count ? list[lane].w : 0;
     int inc = len;
@@ -240,131 +306,158 @@ __device__ __forceinline__ void group_scatter(const DevModel& m, F* cache, const
 }
 
 // ------------------------------------------------------------------ one block
+// A lane's variable: what its decisions need besides the field.
+template <class F>
+struct BlockLane {
+    int k, lo, row, len;
+    uint32_t width;      // 0 beyond the last variable
+    unsigned nbr;        // earlier lanes of the block that share a term with this one
+    int lvl;             // width of its dependency level
+    uint32_t zo;
+    F d;
+    Words4 x;
+    long long z, prop;   // prop: the proposed value where it does not depend on the field
+    bool opt;            // optimal-transition proposal
+};
+
+// Block b's records, random words and proposals: nothing here waits for the
+// changes of earlier blocks.  The next block's records and couplings are
+// prefetched into L1 (couplings: one 128-byte line per variable, two for int64).
+template <class F, class Z, int RULE>
+__device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* zs, int b, int s, int r, float ratio,
+                                                   int lane) {
+    const DevModel& m = a.m;
+    BlockLane<F> q;
+    q.k = b * 32 + lane;
+    int4 x0 = make_int4(0, 0, 0, 0), x1 = x0;
+    q.nbr = 0;
+    q.zo = 0;
+    if (q.k < m.n) {
+        const int4* p = reinterpret_cast<const int4*>(m.idx_rec + q.k);
+        x0 = __ldg(p);
+        x1 = __ldg(p + 1);
+        q.nbr = __ldg(m.blk_mask + q.k);
+        q.zo = (uint32_t)zs[q.k];
+    }
+    const int kn = q.k + 32;
+    if (kn < m.n) {
+        prefetch_l1(m.idx_rec + kn);
+        prefetch_l1(m.blk_mask + kn);
+#pragma unroll
+        for (int o = 0; o < (int)sizeof(F) / 4; ++o) prefetch_l1(Coef<F>::blk(m) + (size_t)kn * 32 + 16 * o);
+    }
+    q.lo = x0.y;
+    q.width = (uint32_t)x0.z;
+    q.row = x0.w;
+    q.len = x1.x;
+    q.lvl = x1.y;
+    if constexpr (Num<F>::is_float) q.d = __uint_as_float((uint32_t)x1.z);
+    else q.d = (long long)(((unsigned long long)(uint32_t)x1.w << 32) | (uint32_t)x1.z);
+    q.x = philox4x32_10((uint32_t)q.k, (uint32_t)s, (uint32_t)r, a.inst, a.key0, a.key1);
+    q.z = (long long)q.lo + (long long)q.zo;
+    q.prop = q.z;
+    q.opt = false;
+    if (RULE != RULE_HEAT_BATH && q.width != 0u) {
+        if (RULE == RULE_OPT) q.opt = unit_open_right(q.x.x2) < ratio;
+        if (!q.opt) {
+            const uint32_t j = pick_below(q.x.x0, q.width);
+            q.prop = (long long)q.lo + (long long)(j >= q.zo ? j + 1u : j);
+        }
+    }
+    return q;
+}
+
 // Decides block b (warp-collective) from the lanes' fields; on return f holds
 // every change of the block, the list its commits.  Returns their number.
 template <class F, class Z, int RULE>
-__device__ __forceinline__ int decide_block(const SweepArgs& a, Z* zs, F& f, Commit* list, int b, int s, int r,
-                                            float beta, float temp, float ratio, int lane, SweepAcc<F>& acc) {
+__device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<F>& q, Z* zs, F& f, Commit* list, int b,
+                                            int s, int r, float beta, float temp, int lane, SweepAcc<F>& acc) {
     constexpr unsigned full = 0xffffffffu;
     const DevModel& m = a.m;
-    const int kb = b * 32, k = kb + lane;
-    const bool on = k < m.n;
-    int4 x0 = make_int4(0, 0, 0, 0), x1 = x0;
-    unsigned nbr = 0;   // earlier lanes of the block that share a term with this one
-    if (on) {
-        const int4* p = reinterpret_cast<const int4*>(m.idx_rec + k);
-        x0 = __ldg(p);
-        x1 = __ldg(p + 1);
-        nbr = __ldg(m.blk_mask + k);
-        // the block's coupling rows, one 128-byte line each (two for int64)
-#pragma unroll
-        for (int o = 0; o < (int)sizeof(F) / 4; ++o) prefetch_l1(Coef<F>::blk(m) + (size_t)k * 32 + 16 * o);
-    }
-    const int lo = x0.y;
-    const uint32_t width = on ? (uint32_t)x0.z : 0u;
-    F d;
-    if constexpr (Num<F>::is_float) d = __uint_as_float((uint32_t)x1.z);
-    else d = (long long)(((unsigned long long)(uint32_t)x1.w << 32) | (uint32_t)x1.z);
-    const Words4 x = philox4x32_10((uint32_t)k, (uint32_t)s, (uint32_t)r, a.inst, a.key0, a.key1);
-    const uint32_t zo = on ? (uint32_t)zs[k] : 0u;
-    const long long z = (long long)lo + (long long)zo;
-    const F* const blk = Coef<F>::blk(m) + (size_t)kb * 32 + lane;   // row p of the block: blk[32 p]
-    long long v = z;
+    const F* const blk = Coef<F>::blk(m) + (size_t)b * 1024 + lane;   // row p of the block: blk[32 p]
+    const long long z = q.z;
+    long long v = z, prop = q.prop;
     int count = 0;
-    auto trace = [&]() {
-        if (a.trace != nullptr && r < a.trace_R && on)
-            a.trace[((size_t)s * a.trace_R + r) * m.n + k] = (int32_t)v;
-    };
-    if constexpr (RULE == RULE_HEAT_BATH) {
-        // one variable after the other, its range split over the lanes
-        const int top = min(32, m.n - kb);
-        for (int p = 0; p < top; ++p) {
-            const uint32_t wp = __shfl_sync(full, width, p);
-            if (wp == 0u) continue;
+    // heat bath: narrow ranges are decided by the lanes (rounds, like the other
+    // rules) unless most of the last block changed; other ranges one variable
+    // after the other by the whole warp
+    bool in_turn = false;
+    if constexpr (RULE == RULE_HEAT_BATH)
+        in_turn = m.max_width >= (Num<F>::is_float ? 64u : 32u) || acc.busy > kBusyBlock;
+    if (RULE == RULE_HEAT_BATH && in_turn) {
+        // the scalar or the warp-wide sum, whichever the level order takes for
+        // the variable's level (the sums differ in their last bits)
+        const unsigned wide = __ballot_sync(full, hb_warp_mode(q.lvl, a.hb_tpr, m.max_width,
+                                                               Num<F>::is_float && m.max_width < 256u));
+        unsigned left = __ballot_sync(full, q.width != 0u);
+        while (left) {
+            const int p = __ffs(left) - 1;
+            left &= left - 1u;
+            const F w = __ldg(blk + 32 * p);
             VarView<F, KIND_QUIO> vv;
             vv.f = __shfl_sync(full, f, p);
-            vv.d = __shfl_sync(full, d, p);
-            const long long zp = __shfl_sync(full, z, p);
-            const long long lp = __shfl_sync(full, lo, p);
-            const uint32_t xp = __shfl_sync(full, x.x0, p);
-            const bool fast = Num<F>::is_float && wp < 256u && lp > -(1 << 22) && lp + (long long)wp < (1 << 22);
-            // the scalar or the warp-wide sum, whichever the level order takes
-            // for this variable's level (the sums differ in their last bits)
-            const bool wide = hb_warp_mode(__shfl_sync(full, x1.y, p), a.hb_tpr, m.max_width,
-                                           Num<F>::is_float && m.max_width < 256u);
-            long long vp;
-            if (vv.linear()) {
-                vp = heat_bath_linear(Num<F>::to_f(vv.lin_coef()), lp, wp, xp, beta);
-            } else if (wide) {
-                vp = heat_bath_warp<F, KIND_QUIO>(vv, zp, lp, wp, xp, beta, lane);
-            } else {
-                bool done = false;
-                vp = zp;
-                if constexpr (Num<F>::is_float) {
-                    if (fast) {
-                        vp = heat_bath_small_warp((float)vv.f, (float)vv.d, zp, lp, wp, xp, beta, temp, lane);
-                        done = true;
-                    }
-                }
-                if (!done) {
-                    vp = wp < kChainValues ? heat_bath_chain<F>(vv, zp, lp, wp, xp, beta, lane)
-                                  : heat_bath_general<F, KIND_QUIO>(vv, zp, lp, wp, xp, beta);
-                }
-            }
-            if (lane == p) v = vp;
+            vv.d = __shfl_sync(full, q.d, p);
+            const uint32_t wp = __shfl_sync(full, q.width, p);
+            const int lp = __shfl_sync(full, q.lo, p);
+            const int zp = lp + (int)__shfl_sync(full, q.zo, p);
+            const int vp = heat_bath_in_turn<F>(vv.f, vv.d, zp, lp, wp, __shfl_sync(full, q.x.x0, p), beta, temp, lane,
+                                                (wide >> p) & 1u);
             if (vp != zp) {
-                const F dp = vv.delta(zp, vp);
-                const int dz = (int)(vp - zp);
-                if constexpr (Num<F>::is_float) acc.de += lane == 0 ? (float)dp : 0.f;
-                else acc.e += lane == 0 ? dp : 0;
+                const int dz = vp - zp;
+                if (lane == 0) {
+                    const F dp = vv.delta(zp, vp);
+                    if constexpr (Num<F>::is_float) acc.de = __fadd_rn(acc.de, (float)dp);   // (no fused multiply-add)
+                    else acc.e += dp;
+                }
                 if (lane == p) {
-                    list[count] = make_int4(k, dz, x0.w, x1.x);
-                    zs[k] = (Z)(v - (long long)lo);
+                    v = vp;
+                    list[count] = make_int4(q.k, dz, q.row, q.len);
+                    zs[q.k] = (Z)(vp - lp);
                     ++acc.changes;
                 } else {
-                    solo_add(&f, __ldg(blk + 32 * p), dz);
+                    solo_add(&f, w, dz);
                 }
                 ++count;
             }
         }
-        trace();
-        return count;
     } else {
-        long long prop = z;
-        bool opt = false;
-        if (width != 0u) {
-            if (RULE == RULE_OPT) opt = unit_open_right(x.x2) < ratio;
-            if (!opt) {
-                const uint32_t j = pick_below(x.x0, width);
-                prop = (long long)lo + (long long)(j >= zo ? j + 1u : j);
-            }
-        }
-        unsigned open = __ballot_sync(full, width != 0u);   // lanes still to be decided
+        unsigned open = __ballot_sync(full, q.width != 0u);   // lanes still to be decided
         while (open) {
-            const bool mine = (open >> lane) & 1u;
             F de = F(0);
             bool chg = false;
-            if (mine) {
-                if (RULE == RULE_OPT && opt) {
-                    VarView<F, KIND_QUIO> vv;
-                    vv.f = f;
-                    vv.d = d;
-                    prop = opt_argmin<F, KIND_QUIO>(vv, z, lo, (long long)lo + (long long)width);
+            if ((open >> lane) & 1u) {
+                VarView<F, KIND_QUIO> vv;
+                vv.f = f;
+                vv.d = q.d;
+                if constexpr (RULE == RULE_HEAT_BATH) {
+                    if (vv.linear()) prop = heat_bath_linear(Num<F>::to_f(f), q.lo, q.width, q.x.x0, beta);
+                    else if constexpr (Num<F>::is_float) {
+                        if (q.lo > -(1 << 22) && (long long)q.lo + (long long)q.width < (1 << 22))
+                            prop = heat_bath_quio_f32_small((float)f, (float)q.d, z, q.lo, q.width, q.x.x0, beta, temp);
+                        else
+                            prop = heat_bath_general<F, KIND_QUIO>(vv, z, q.lo, q.width, q.x.x0, beta);
+                    } else {
+                        prop = heat_bath_narrow(vv, z, q.lo, q.width, q.x.x0, beta, m.max_width);
+                    }
+                    chg = prop != z;
+                    if (chg) de = vv.delta(z, prop);
+                } else {
+                    if (RULE == RULE_OPT && q.opt)
+                        prop = opt_argmin<F, KIND_QUIO>(vv, z, q.lo, (long long)q.lo + (long long)q.width);
+                    de = quio_delta<F>(f, q.d, z, prop);
+                    chg = prop != z && metropolis_accept<F>(de, q.x.x1, beta);
                 }
-                de = quio_delta<F>(f, d, z, prop);
-                chg = prop != z && metropolis_accept<F>(de, x.x1, beta);
             }
             const unsigned c = __ballot_sync(full, chg);
             if (!c) break;
             // the first lane whose field one of the changes reaches decides again
-            const unsigned late = __ballot_sync(full, mine && (nbr & c) != 0u);
-            const int q = late ? __ffs(late) - 1 : 32;
-            const unsigned done = late ? (1u << q) - 1u : full;
+            const unsigned late = __ballot_sync(full, ((open >> lane) & 1u) && (q.nbr & c) != 0u);
+            const unsigned done = late ? (late & (0u - late)) - 1u : full;
             unsigned com = c & done;
-            if (chg && ((com >> lane) & 1u)) {
+            if ((com >> lane) & 1u) {
                 v = prop;
-                list[count + __popc(com & ((1u << lane) - 1u))] = make_int4(k, (int)(v - z), x0.w, x1.x);
-                zs[k] = (Z)(v - (long long)lo);
+                list[count + __popc(com & ((1u << lane) - 1u))] = make_int4(q.k, (int)(v - z), q.row, q.len);
+                zs[q.k] = (Z)(v - (long long)q.lo);
                 ++acc.changes;
                 if constexpr (!Num<F>::is_float) acc.e += de;
             }
@@ -378,14 +471,16 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, Z* zs, F& f, Com
                 if (lane != p) solo_add(&f, w, dp);
                 if constexpr (Num<F>::is_float) {   // summed in the visiting order, by one lane
                     const float ep = __shfl_sync(full, (float)de, p);
-                    acc.de += lane == 0 ? ep : 0.f;
+                    if (lane == 0) acc.de = __fadd_rn(acc.de, ep);
                 }
             }
             open &= ~done;
         }
-        trace();
-        return count;
     }
+    if constexpr (RULE == RULE_HEAT_BATH) acc.busy = count;
+    if (a.trace != nullptr && r < a.trace_R && q.k < m.n)
+        a.trace[((size_t)s * a.trace_R + r) * m.n + q.k] = (int32_t)v;
+    return count;
 }
 
 // ------------------------------------------------------------------ one sweep
@@ -416,31 +511,34 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
             const int np = acc.last >= 0 ? ctl[acc.par ^ 1] : 0;
             if (t < 32) {
                 const int k = b * 32 + lane;
-                F f = F(0);
-                if (k < m.n) {
-                    f = cache[k];
-                    if (acc.last != b) f = add_commits<F>(m, f, prev, np, k);
+                const int ahead = acc.last != b ? np : 0;
+                F f[1] = {k < m.n ? cache[k] : F(0)};
+                // the first rows of the last block's changes are on their way
+                // while this block's random words are made
+                const int j[1] = {k < m.n ? k : -1};
+                RowPart<F, 1> rows;
+                load_rows<F, 1>(rows, m, prev, 0, ahead, j);
+                const BlockLane<F> q = block_lane<F, Z, RULE>(a, zs, b, s, r, ratio, lane);
+                add_rows<F, 1>(rows, prev, 0, ahead, f);
+                for (int c = kRows<F>; c < ahead; c += kRows<F>) {
+                    load_rows<F, 1>(rows, m, prev, c, ahead, j);
+                    add_rows<F, 1>(rows, prev, c, ahead, f);
                 }
-                const int cnt = decide_block<F, Z, RULE>(a, zs, f, lists + 32 * acc.par, b, s, r, beta, temp, ratio,
+                const int cnt = decide_block<F, Z, RULE>(a, q, zs, f[0], lists + 32 * acc.par, b, s, r, beta, temp,
                                                          lane, acc);
-                if (k < m.n) cache[k] = f;
+                if (k < m.n) cache[k] = f[0];
                 if (lane == 0) ctl[acc.par] = cnt;
             }
             if (np > 0 && (t >= 32 || tpr == 32)) {
-                const int nt = tpr > 32 ? tpr - 32 : 32;
-                for (int j = tpr > 32 ? t - 32 : t; j < m.n; j += nt) {
-                    const int bj = j >> 5;
-                    if (bj != b && bj != acc.last) cache[j] = add_commits<F>(m, cache[j], prev, np, j);
-                }
+                const int skip = tpr > 32 ? 32 : 0;
+                add_commits<F, MEM>(m, cache, prev, np, acc.last, b, t - skip, tpr - skip);
             }
             named_bar(bar_id, tpr);
             acc.par ^= 1;
             acc.last = b;
         }
         if (flush) {
-            const int np = ctl[acc.par ^ 1];
-            for (int j = t; j < m.n; j += tpr)
-                if ((j >> 5) != acc.last) cache[j] = add_commits<F>(m, cache[j], lists + 32 * (acc.par ^ 1), np, j);
+            add_commits<F, MEM>(m, cache, lists + 32 * (acc.par ^ 1), ctl[acc.par ^ 1], acc.last, acc.last, t, tpr);
             named_bar(bar_id, tpr);
             acc.last = -1;
         }
@@ -452,7 +550,8 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
             for (int b = 0; b < nb; ++b) {
                 const int k = b * 32 + lane;
                 F f = k < m.n ? cache[k] : F(0);
-                const int cnt = decide_block<F, Z, RULE>(a, zs, f, lists, b, s, r, beta, temp, ratio, lane, acc);
+                const BlockLane<F> q = block_lane<F, Z, RULE>(a, zs, b, s, r, ratio, lane);
+                const int cnt = decide_block<F, Z, RULE>(a, q, zs, f, lists, b, s, r, beta, temp, lane, acc);
                 if (k < m.n) cache[k] = f;
                 __syncwarp();
                 if (cnt == 0 || nb == 1) continue;
