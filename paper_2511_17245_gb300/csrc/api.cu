@@ -254,11 +254,18 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
     dm.n = n;
     dm.is_float = M->is_float ? 1 : 0;
     dm.max_width = M->max_width;
+    dm.z_base = lo[0];
+    int64_t z_top = upper[0];
+    for (int32_t k = 0; k < n; ++k) {
+        dm.z_base = std::min(dm.z_base, lo[k]);
+        z_top = std::max(z_top, upper[k]);
+    }
+    dm.z_span = (uint32_t)(z_top - dm.z_base);
     dm.const_i = (int64_t)const_i;
     dm.const_d = const_d;
     struct Offs {
         size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk = 0;
-        size_t adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
+        size_t up_rec, adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
         size_t slot_base, omega, aconst_i, aconst_f, aconst_d, inc_term, inc_exp, inc_rec, term_ptr, mem_var, mem_exp,
             tcoef_i, tcoef_f, tcoef_d;
     } off{};
@@ -361,6 +368,21 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         off.lvl_vars = blob.add(lvl_vars);
         off.lvl_rec = blob.add(rec);
         off.adj_col = blob.add(col);
+        std::vector<int32_t> up(4 * (size_t)n, 0), up_first(n), up_order(n);
+        for (int32_t k = 0; k < n; ++k) {
+            up_first[k] =
+                (int32_t)(std::upper_bound(col.begin() + ptr[k], col.begin() + ptr[k] + deg[k], k) - col.begin());
+            up_order[k] = k;
+        }
+        auto up_key = [&](int32_t k) { return (ptr[k] + deg[k] - up_first[k]) * 4 + (up_first[k] & 3); };
+        std::stable_sort(up_order.begin(), up_order.end(), [&](int32_t x, int32_t y) { return up_key(x) > up_key(y); });
+        for (int32_t i = 0; i < n; ++i) {
+            const int32_t k = up_order[i];
+            up[4 * (size_t)i] = k;
+            up[4 * (size_t)i + 1] = up_first[k];
+            up[4 * (size_t)i + 2] = (int32_t)(ptr[k] + deg[k]);
+        }
+        off.up_rec = blob.add(up);
         if (sa::plan_block_model(n, M->n_levels)) {
             // blocked sweeps: records in index order, the earlier neighbours in
             // each variable's block of 32 and the block's couplings
@@ -563,6 +585,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
             else dm.blk_i = at<int64_t>(b, off.blk);
         }
         dm.adj_col = at<int32_t>(b, off.adj_col);
+        dm.up_rec = at<int32_t>(b, off.up_rec);
         if (M->is_float) {
             dm.adj_f = at<float>(b, off.adj_f);
             dm.adj_d = off.adj_d == SIZE_MAX ? nullptr : at<double>(b, off.adj_d);

@@ -3,6 +3,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "sa_internal.h"
 
 namespace sa {
@@ -178,10 +180,170 @@ __global__ void __launch_bounds__(256) energy_kernel(const EnergyArgs a) {
     }
 }
 
+// ------------------------------------------------------------------ QUIO, several states per block
+// E = sum_k z_k (lin_k + diag_k z_k + sum_{j > k} J_kj z_j): each pair once, from
+// the row of its smaller variable (up_rec).  A block stages G states in shared
+// memory, interleaved by variable and in 1, 2 or 4 bytes above z_base, so that
+// one shared load gives z_j of all of them and a row's entries are read once per
+// G states; a thread takes whole rows, four entries per vector load,
+// rows of the same length and alignment side by side (an FP64 instruction holds
+// the pipe for 16 cycles however few lanes want it).
+// What bounds it: FP64 additions (two lanes per cycle and SM), one per pair and
+// state, 0.52 ms for 4096 states of 80,000 pairs; the conversions to FP64, which
+// share that pipe, are done by moving bits.  The one-state-per-block form walked
+// every pair from both ends with a 4-byte gather from global memory each and
+// waited for the load queue (6.9 ms).
+__device__ __forceinline__ double widen_f(float x) {
+    const uint32_t u = __float_as_uint(x);
+    const uint32_t e = (u >> 23) & 0xFFu;
+    if (e - 1u >= 254u) return (double)x;   // zero, denormal, infinite, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+template <class Z>
+__device__ __forceinline__ double widen_z(int z) {
+    if constexpr (sizeof(Z) < 4) return z == 0 ? 0.0 : widen_f(__int2float_rn(z));   // (below 2^24: see launch_energy)
+    else return __int2double_rn(z);
+}
+
+template <class Z, int G>
+struct alignas(sizeof(Z) * G) ZPack {
+    Z z[G];
+};
+
+template <bool IS_FLOAT, class Z, int G>
+__global__ void __launch_bounds__(256) quio_energy_kernel(const EnergyArgs a) {
+    using Acc = typename std::conditional<IS_FLOAT, double, long long>::type;
+    extern __shared__ __align__(16) uint8_t zraw[];
+    __shared__ Acc red[8];
+    ZPack<Z, G>* zs = reinterpret_cast<ZPack<Z, G>*>(zraw);
+    const DevModel& m = a.m;
+    const int64_t s0 = (int64_t)blockIdx.x * G;
+    const int ns = (int)min((int64_t)G, a.n_states - s0);
+    // stage, with the bounds check: a value outside [l_k, u_k] is reported
+    for (int k = threadIdx.x; k < m.n; k += blockDim.x) {
+        const VarMeta mt = m.meta[k];
+        ZPack<Z, G> q;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            long long zk = mt.lo;
+            if (g < ns) {
+                zk = a.states[(s0 + g) * m.n + k];
+                if (zk < mt.lo || zk > (long long)mt.lo + (long long)mt.width) {
+                    atomicExch(a.bad, 1);
+                    zk = mt.lo;
+                }
+            }
+            q.z[g] = (Z)(uint32_t)(zk - m.z_base);
+        }
+        zs[k] = q;
+    }
+    __syncthreads();
+    Acc e[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) e[g] = Acc(0);
+    for (int i = threadIdx.x; i < m.n; i += blockDim.x) {
+        const int4 rec = __ldg(reinterpret_cast<const int4*>(m.up_rec) + i);
+        const int k = rec.x, first = rec.y, end = rec.z;
+        Acc f[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            if constexpr (IS_FLOAT) f[g] = m.lin_d[k];
+            else f[g] = m.lin_i[k];
+        }
+        for (int q0 = first & ~3; q0 < end; q0 += 4) {
+            const int4 c4 = __ldg(reinterpret_cast<const int4*>(m.adj_col + q0));
+            const int col[4] = {c4.x, c4.y, c4.z, c4.w};
+            Acc w[4];
+            if constexpr (IS_FLOAT) {
+                if (m.adj_d != nullptr) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) w[u] = __ldg(m.adj_d + q0 + u);
+                } else {
+                    const float4 w4 = __ldg(reinterpret_cast<const float4*>(m.adj_f + q0));
+                    w[0] = widen_f(w4.x); w[1] = widen_f(w4.y); w[2] = widen_f(w4.z); w[3] = widen_f(w4.w);
+                }
+            } else {
+                const longlong2* wp = reinterpret_cast<const longlong2*>(m.adj_i + q0);
+                const longlong2 wa = __ldg(wp), wb = __ldg(wp + 1);
+                w[0] = wa.x; w[1] = wa.y; w[2] = wb.x; w[3] = wb.y;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (q0 + u < first || q0 + u >= end) continue;
+                const ZPack<Z, G> zj = zs[col[u]];
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int z = m.z_base + (int)(uint32_t)zj.z[g];
+                    if constexpr (IS_FLOAT) f[g] += w[u] * widen_z<Z>(z);
+                    else f[g] += w[u] * (long long)z;
+                }
+            }
+        }
+        const ZPack<Z, G> zk = zs[k];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            const int z = m.z_base + (int)(uint32_t)zk.z[g];
+            if constexpr (IS_FLOAT) {
+                const double zd = widen_z<Z>(z);
+                e[g] += zd * (f[g] + m.diag_d[k] * zd);
+            } else {
+                e[g] += (long long)z * (f[g] + m.diag_i[k] * (long long)z);
+            }
+        }
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        const Acc tot = block_sum<Acc>(e[g], red);
+        if (threadIdx.x == 0 && g < ns) {
+            if constexpr (IS_FLOAT) reinterpret_cast<double*>(a.energies)[s0 + g] = m.const_d + tot;
+            else reinterpret_cast<long long*>(a.energies)[s0 + g] = m.const_i + tot;
+        }
+        __syncthreads();
+    }
+}
+
+template <bool IS_FLOAT, class Z, int G>
+int launch_quio_energy(const EnergyArgs& a, cudaStream_t st) {
+    auto kern = quio_energy_kernel<IS_FLOAT, Z, G>;
+    const size_t sh = (size_t)a.m.n * sizeof(Z) * G;
+    if (sh > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+        if (e != cudaSuccess) return (int)e;
+    }
+    kern<<<(unsigned)((a.n_states + G - 1) / G), 256, sh, st>>>(a);
+    return (int)cudaGetLastError();
+}
+
+// Four states per block when that still gives every SM a few blocks and they
+// fit, else one; returns false when one state does not fit on chip.
+template <bool IS_FLOAT, class Z>
+bool quio_energy_shape(const EnergyArgs& a, cudaStream_t st, int& rc) {
+    const size_t room = (size_t)sweep_max_shared_optin() - 1024, one = (size_t)a.m.n * sizeof(Z);
+    if (4 * one <= room && a.n_states >= 4 * 304) rc = launch_quio_energy<IS_FLOAT, Z, 4>(a, st);
+    else if (one <= room) rc = launch_quio_energy<IS_FLOAT, Z, 1>(a, st);
+    else return false;
+    return true;
+}
+template <bool IS_FLOAT>
+bool quio_energy(const EnergyArgs& a, cudaStream_t st, int& rc) {
+    const uint32_t span = a.m.z_span;
+    const long long lo = a.m.z_base, hi = lo + (long long)span;
+    const bool small = lo > -(1 << 24) && hi < (1 << 24);   // exact in fp32 on the way to FP64
+    if (small && span <= 0xFFu) return quio_energy_shape<IS_FLOAT, uint8_t>(a, st, rc);
+    if (small && span <= 0xFFFFu) return quio_energy_shape<IS_FLOAT, uint16_t>(a, st, rc);
+    return quio_energy_shape<IS_FLOAT, uint32_t>(a, st, rc);
+}
+
 }  // namespace
 
 int launch_energy(const EnergyArgs& a, void* stream) {
     if (a.n_states <= 0) return 0;
+    if (a.m.kind == KIND_QUIO) {
+        int rc = 0;
+        const bool done = a.m.is_float ? quio_energy<true>(a, (cudaStream_t)stream, rc)
+                                       : quio_energy<false>(a, (cudaStream_t)stream, rc);
+        if (done) return rc;
+    }
     const unsigned grid = (unsigned)a.n_states;
     if (a.m.is_float) energy_kernel<true><<<grid, 256, 0, (cudaStream_t)stream>>>(a);
     else energy_kernel<false><<<grid, 256, 0, (cudaStream_t)stream>>>(a);

@@ -55,6 +55,12 @@ struct DevModel {
 
     // QUIO (every term of total degree <= 2):
     //   E = c + sum_k lin_k z_k + sum_k diag_k z_k^2 + sum_{i<j} J_ij z_i z_j
+    // [n]: {k, first entry of row k with a column above k, end of row k, 0}, by
+    // the number of those entries (descending) and the first one's place in its
+    // group of four, so that a warp's lanes walk alike
+    const int32_t* up_rec;
+    int32_t z_base;             // smallest lower bound
+    uint32_t z_span;            // largest upper bound minus z_base
     const int32_t* adj_col;     // symmetric adjacency, both directions
     const int64_t* adj_i;
     const float* adj_f;
