@@ -264,9 +264,10 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
     dm.const_i = (int64_t)const_i;
     dm.const_d = const_d;
     struct Offs {
-        size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk = 0;
+        size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk_w = 0, blk_i = 0;
+        bool blk_wide = false;
         size_t up_rec, adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
-        size_t slot_base, omega, aconst_i, aconst_f, aconst_d, inc_term, inc_exp, inc_rec, term_ptr, mem_var, mem_exp,
+        size_t slot_base, omega, aconst_i, aconst_f, aconst_d, inc_term, inc_exp, inc_rec, inc16 = SIZE_MAX, term_ptr, mem_var, mem_exp,
             tcoef_i, tcoef_f, tcoef_d;
     } off{};
     std::vector<int32_t> lvl_ptr, lvl_vars;
@@ -394,20 +395,28 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
                 }
             std::vector<uint32_t> mask(n, 0);
             const size_t cells = (size_t)((n + 31) / 32) * 32 * 32;
+            std::vector<int32_t> bw(cells, 0);
             std::vector<int64_t> bi(M->is_float ? 0 : cells, 0);
-            std::vector<float> bf(M->is_float ? cells : 0, 0.f);
             for (int32_t k = 0; k < n; ++k) {
                 const int32_t kb = k / 32 * 32;
                 auto first = std::lower_bound(col.begin() + ptr[k], col.begin() + ptr[k] + deg[k], kb);
                 for (int64_t e = first - col.begin(); e < ptr[k] + deg[k] && col[e] < kb + 32; ++e) {
                     if (col[e] < k) mask[k] |= 1u << (col[e] - kb);
-                    if (M->is_float) bf[(size_t)k * 32 + (col[e] - kb)] = (float)vd[e];
-                    else bi[(size_t)k * 32 + (col[e] - kb)] = vi[e];
+                    const size_t at = (size_t)k * 32 + (col[e] - kb);
+                    if (M->is_float) {
+                        const float w = (float)vd[e];
+                        std::memcpy(&bw[at], &w, 4);
+                    } else {
+                        bi[at] = vi[e];
+                        bw[at] = (int32_t)vi[e];
+                        if (bw[at] != vi[e]) off.blk_wide = true;
+                    }
                 }
             }
             off.idx_rec = blob.add(ir);
             off.blk_mask = blob.add(mask);
-            off.blk = M->is_float ? blob.add(bf) : blob.add(bi);
+            off.blk_w = blob.add(bw);
+            if (off.blk_wide) off.blk_i = blob.add(bi);
         }
         if (M->is_float) {
             std::vector<float> vf(vd.size()), lf(n), df(n);
@@ -428,7 +437,9 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         for (auto& t : terms)
             for (auto& m : t.mem) omega[m.var] |= (1ull << m.exp);
         std::vector<int32_t> slot_base(n + 1, 0);
-        for (int32_t k = 0; k < n; ++k) slot_base[k + 1] = slot_base[k] + __builtin_popcountll(omega[k]);
+        // (multilinear models: one slot per variable, used or not, so that slot = variable)
+        for (int32_t k = 0; k < n; ++k)
+            slot_base[k + 1] = slot_base[k] + (multilinear ? 1 : __builtin_popcountll(omega[k]));
         const int32_t n_slots = slot_base[n];
         auto slot_of = [&](int32_t k, int32_t e) {
             return slot_base[k] + __builtin_popcountll((omega[k] & ((1ull << e) - 1ull)) >> 1);
@@ -508,6 +519,22 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
                 q[2] = inc_exp[e] | (c << 8) | (ones ? 1 << 16 : 0);
                 q[3] = packed;
             }
+        // the compact form (DevModel::inc16)
+        bool compact = multilinear && n <= 65534 && max_order <= 4 && dm.z_span <= (uint32_t)INT32_MAX;
+        for (int32_t k = 0; k < n && compact; ++k) compact = lo[k] == dm.z_base;
+        if (!M->is_float)
+            for (int32_t tt = 0; tt < n_iterms && compact; ++tt) compact = tcoef_i[tt] == (int64_t)(int32_t)tcoef_i[tt];
+        std::vector<int32_t> inc16(compact ? (size_t)iptr[n] * 4 : 0, 0);
+        if (compact)
+            for (size_t e = 0; e < (size_t)iptr[n]; ++e) {
+                const int32_t* q = inc_rec.data() + e * 16;
+                const int32_t no = (q[2] >> 8) & 0xFF;
+                uint32_t v[3];
+                for (int c = 0; c < 3; ++c) v[c] = c < no ? (uint32_t)q[4 + c] : 0xFFFFu;
+                inc16[4 * e] = q[0];
+                inc16[4 * e + 1] = (int32_t)(v[0] | (v[1] << 16));
+                inc16[4 * e + 2] = (int32_t)v[2];
+            }
         // neighbours for levels: members of incident interaction terms
         nb_ptr.assign(n + 1, 0);
         for (int32_t k = 0; k < n; ++k) {
@@ -548,6 +575,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         off.inc_term = blob.add(inc_term);
         off.inc_exp = blob.add(inc_exp);
         off.inc_rec = blob.add(inc_rec);
+        if (compact) off.inc16 = blob.add(inc16);
         off.term_ptr = blob.add(term_ptr);
         off.mem_var = blob.add(mem_var);
         off.mem_exp = blob.add(mem_exp);
@@ -581,8 +609,8 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         if (sa::plan_block_model(n, M->n_levels)) {
             dm.idx_rec = at<sa::LevelRec>(b, off.idx_rec);
             dm.blk_mask = at<uint32_t>(b, off.blk_mask);
-            if (M->is_float) dm.blk_f = at<float>(b, off.blk);
-            else dm.blk_i = at<int64_t>(b, off.blk);
+            dm.blk_w = at<int32_t>(b, off.blk_w);
+            if (off.blk_wide) dm.blk_i = at<int64_t>(b, off.blk_i);
         }
         dm.adj_col = at<int32_t>(b, off.adj_col);
         dm.up_rec = at<int32_t>(b, off.up_rec);
@@ -601,6 +629,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         dm.inc_term = at<int32_t>(b, off.inc_term);
         dm.inc_exp = at<int32_t>(b, off.inc_exp);
         dm.inc_rec = at<int32_t>(b, off.inc_rec);
+        dm.inc16 = off.inc16 == SIZE_MAX ? nullptr : at<int32_t>(b, off.inc16);
         dm.term_ptr = at<int32_t>(b, off.term_ptr);
         dm.mem_var = at<int32_t>(b, off.mem_var);
         dm.mem_exp = at<int32_t>(b, off.mem_exp);

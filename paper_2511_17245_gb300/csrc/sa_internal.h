@@ -50,8 +50,8 @@ struct DevModel {
     // consecutive variables; null otherwise
     const LevelRec* idx_rec;    // [n]: records in index order, slot_base = width of the variable's level
     const uint32_t* blk_mask;   // [n]: bit j set iff variable 32 (k / 32) + j < k shares a term with k
-    const int64_t* blk_i;       // [32 ceil(n / 32)][32]: J_kj of the variables j of k's block
-    const float* blk_f;
+    const int32_t* blk_w;       // [32 ceil(n / 32)][32]: J_kj of the variables j of k's block (fp32 bits or int32)
+    const int64_t* blk_i;       // the same in int64, when some J_kj does not fit int32 (blk_w is not read then)
 
     // QUIO (every term of total degree <= 2):
     //   E = c + sum_k lin_k z_k + sum_k diag_k z_k^2 + sum_{i<j} J_ij z_i z_j
@@ -89,6 +89,11 @@ struct DevModel {
     // {their variables v1..v3, term}, {their coefficient slots (slot_base[v] +
     // index of the exponent), 0}, {their lower bounds, 0}
     const int32_t* inc_rec;
+    // multilinear models of at most 65,534 variables with one lower bound, terms
+    // of at most 4 members and coefficients that fit 32 bits: the same in one
+    // 16-byte group, {coefficient (int32 or fp32 bits), v1 | v2 << 16, v3, 0} with
+    // 0xFFFF for no variable (variable v's slot is v); null otherwise
+    const int32_t* inc16;
     const int32_t* term_ptr;    // [n_iterms + 1] into mem_var / mem_exp
     const int32_t* mem_var;     // members (distinct variables) of interaction terms
     const int32_t* mem_exp;     // their exponents
@@ -123,9 +128,11 @@ struct SweepArgs {
     uint8_t* gstate;            // per-replica state slabs when not on chip
     int64_t rep_bytes;          // bytes of one replica's state region
     int32_t off_z, off_cache, off_ctl, off_list, off_red;
+    int32_t off_blk;            // blocked sweeps: two staged blocks (kBlockStage bytes each)
     int32_t off_lvl;            // level boundaries staged in the replica region (-1: read from the model)
     int32_t blocked;            // sweep in blocks of 32 variables (the model has idx_rec)
     int32_t hb_tpr;             // threads per replica that decide the form of heat-bath sums (hb_warp_mode)
+    int32_t _pad0;
     int32_t rpc;                // replicas per block
     int32_t tpr;                // threads per replica (multiple of 32)
     int32_t heavy_links;        // link_len above which updates are cooperative
@@ -285,14 +292,34 @@ inline bool plan_blocked(const PlanModel& m, int rule, bool allowed) {
     return rule != RULE_HEAT_BATH || (int64_t)m.n <= (int64_t)kBlockWidthHeat * m.n_levels;
 }
 
+// Bytes of one block staged on chip: couplings (32 x 32 x 4), records, masks.
+constexpr int kBlockStage = 4096 + 32 * (int)sizeof(LevelRec) + 128;
+
 // Threads that a replica of a blocked sweep can use: one warp decides; the
 // others add its changes to the other fields (complete graphs: every field,
 // several rows deep; else the rows' links).
 inline int plan_blocked_threads(const PlanModel& m) {
     if (m.n <= 32) return 32;
-    const int work = m.dense_rows ? m.n / 4 : (4 * m.mean_links < m.n ? 4 * m.mean_links : m.n);
+    // complete graph of 1000 variables, 152 replicas x 50 sweeps: 128 threads
+    // 11.7 ms, 192 7.8, 256 7.0, 384 6.4, 512 7.4
+    if (m.dense_rows) {
+        const int want = (m.n * 3 / 8 + 31) / 32 * 32;
+        return want > 512 ? 512 : (want < 128 && m.n > 64 ? 128 : want);
+    }
+    const int work = 4 * m.mean_links < m.n ? 4 * m.mean_links : m.n;
     const int want = 32 + (work + 31) / 32 * 32;
     return want > 512 ? 512 : want;
+}
+
+// Threads that a replica of a level-by-level sweep can use: twice the mean level
+// width, so that nearly every level is one round (levels of a random graph are
+// up to twice as wide as the mean).  1501 variables of mean degree 16, 36 levels,
+// 512 replicas x 100 sweeps: 32 threads 13.9 ms, 64 9.4, 96 9.0, 128 9.6.
+inline int plan_level_threads(const PlanModel& m, int tpr) {
+    const int levels = m.n_levels > 0 ? m.n_levels : 1;
+    int want = (2 * (m.n / levels) + 31) / 32 * 32;
+    want = want > 256 ? 256 : want;
+    return want > tpr ? want : tpr;
 }
 
 // Per-replica state layout and launch shape of one run.
@@ -305,7 +332,7 @@ struct RunPlan {
     int32_t in_global;          // replica state in global memory instead of shared memory
     int64_t rep_bytes;          // bytes of one replica's state region
     int64_t shared_bytes;       // dynamic shared memory of one block
-    int32_t off_z, off_cache, off_ctl, off_list, off_red, off_lvl;
+    int32_t off_z, off_cache, off_ctl, off_list, off_red, off_lvl, off_blk;
     int32_t blocked, hb_tpr;    // see SweepArgs (set by plan_run)
 };
 
@@ -315,7 +342,8 @@ inline int64_t plan_round16(int64_t x) { return (x + 15) / 16 * 16; }
 // each), the cache (int64 or fp32), the control words (three list counters or
 // the commit counts and commands of a blocked sweep), the cooperative update
 // list or a blocked sweep's two commit lists, the reduction scratch (one 8-byte word
-// per warp) and, when it takes at most 16 KB, the level boundary table.
+// per warp), when it takes at most 16 KB the level boundary table, and for models
+// of blocked sweeps two staged blocks.
 // `zbytes` may exceed the model's own (a batch uses its widest).  QUIO rows are
 // cheap per entry (one atomic) and go inline up to 64 links; HUIO incidences
 // cost a term product each and go inline up to 8.
@@ -334,7 +362,8 @@ inline int64_t plan_layout(const PlanModel& m, int zbytes, int tpr, RunPlan* p) 
     const int64_t off_lvl = plan_round16(p->off_red + (int64_t)(tpr / 32) * 8);
     const bool lvl_on_chip = lvl_bytes <= 16384;
     p->off_lvl = lvl_on_chip ? (int32_t)off_lvl : -1;
-    p->rep_bytes = plan_round16(off_lvl + (lvl_on_chip ? lvl_bytes : 0));
+    p->off_blk = (int32_t)plan_round16(off_lvl + (lvl_on_chip ? lvl_bytes : 0));
+    p->rep_bytes = p->off_blk + (m.block_model ? 2 * kBlockStage : 0);
     return p->rep_bytes;
 }
 
@@ -387,9 +416,9 @@ inline const char* plan_run(const PlanModel& m, int rule, bool allow_blocks, int
     // (the shape does not depend on allow_blocks, so that float energies, summed
     // in FP64 over the replica's threads, are the same bits either way)
     const bool blocked = plan_blocked(m, rule, true);
-    if (blocked && tpr_req <= 0) {
+    if (tpr_req <= 0) {
         const int rpc = p->rpc;
-        int tpr = plan_blocked_threads(m);
+        int tpr = blocked ? plan_blocked_threads(m) : plan_level_threads(m, p->tpr);
         const int cap = 512 / rpc / 32 * 32;
         tpr = tpr > cap ? cap : tpr;
         RunPlan q{};
@@ -466,6 +495,7 @@ inline void plan_apply(const RunPlan& p, SweepArgs& a) {
     a.off_list = p.off_list;
     a.off_red = p.off_red;
     a.off_lvl = p.off_lvl;
+    a.off_blk = p.off_blk;
     a.rpc = p.rpc;
     a.tpr = p.tpr;
     a.heavy_links = p.heavy_links;

@@ -13,8 +13,8 @@
 // added to a field in that order, and nothing but warp shuffles separates two
 // changes of a block.  Changes reach the other fields block by block.
 //
-// What bounds it: the chain of rounds, about 200 cycles each (decision, two
-// ballots, one coupling row from L1).  Deciding level by level, or a window of
+// What bounds it: the chain of rounds (decision, two ballots, one coupling row
+// from shared memory).  Deciding level by level, or a window of
 // levels up to its first change, cost two group barriers, a Philox block and an
 // L2 row per change instead (about 2500 cycles).
 #pragma once
@@ -30,6 +30,7 @@ struct SweepAcc {
     float de;                        // float models: energy changes since the last fold into e
     float drift;                     // float models: largest error of a field seen by a refresh
     int busy;                        // heat bath: changes of the last block
+    int turn;                        // blocks begun: which staged place is current
     int par;                         // blocked sweeps: which of the two commit lists is current
     int last;                        // and the block whose changes are not applied everywhere yet (-1: none)
 };
@@ -167,68 +168,88 @@ __device__ __noinline__ int heat_bath_in_turn(F f, F d, int z, int lo, uint32_t 
     return (int)heat_bath_general<F, KIND_QUIO>(vv, z, lo, width, xu, beta);
 }
 
-// ------------------------------------------------------------------ changes to the other fields
-// A pointer into shared memory whose address space the compiler can see (for
-// functions out of line, which are given generic pointers).
-template <int MEM, class T>
-__device__ __forceinline__ T* in_shared(T* p) {
-    if constexpr (MEM == MEM_SHARED) return static_cast<T*>(__cvta_shared_to_generic(__cvta_generic_to_shared(p)));
-    else return p;
+// A lane's own variable, narrow range (out of line for the same reason).
+template <class F>
+__device__ __noinline__ int heat_bath_lane(F f, F d, int z, int lo, uint32_t width, uint32_t xu, float beta, float temp,
+                                           uint32_t max_width) {
+    VarView<F, KIND_QUIO> vv;
+    vv.f = f;
+    vv.d = d;
+    if (vv.linear()) return (int)heat_bath_linear(Num<F>::to_f(f), lo, width, xu, beta);
+    if constexpr (Num<F>::is_float) {
+        if (lo > -(1 << 22) && (long long)lo + (long long)width < (1 << 22))
+            return (int)heat_bath_quio_f32_small((float)f, (float)d, z, lo, width, xu, beta, temp);
+        return (int)heat_bath_general<F, KIND_QUIO>(vv, z, lo, width, xu, beta);
+    } else {
+        return (int)heat_bath_narrow(vv, z, lo, width, xu, beta, max_width);
+    }
 }
 
+// ------------------------------------------------------------------ changes to the other fields
 // Fields of a complete graph: the commits' couplings to field j, in order.  Row
 // k lists every j != k in order, so entry j - [j > k] of the row is J_kj.  Rows
-// are read past L1 (each entry is used once), kRows at a time and for NF fields
-// at a time, all loads before the first addition.
-template <class F>
-constexpr int kRows = Num<F>::is_float ? 8 : 4;
-template <class F, int NF>
+// are read past L1 (each entry is used once), NR at a time and for NF fields at a
+// time, all loads before the first addition.
+// (Predicates instead of branches throughout: a uniform branch per row costs
+// more than the row.)
+template <class F, int NF, int NR>
 struct RowPart {
-    F w[NF][kRows<F>];
+    F w[NF][NR];
+    int dz[NR];          // 0 beyond the last commit
 };
-template <class F, int NF>
-__device__ __forceinline__ void load_rows(RowPart<F, NF>& q, const DevModel& m, const Commit* list, int c, int count,
+template <class F, int NF, int NR>
+__device__ __forceinline__ void load_rows(RowPart<F, NF, NR>& q, const DevModel& m, const Commit* list, int c, int count,
                                           const int (&j)[NF]) {
 #pragma unroll
-    for (int u = 0; u < kRows<F>; ++u)
-        if (c + u < count) {
-            const Commit e = list[c + u];
+    for (int u = 0; u < NR; ++u) {
+        const Commit e = list[(c + u) & 31];   // (entries beyond the count are read and not used)
+        const bool on = c + u < count;
+        q.dz[u] = on ? e.y : 0;
 #pragma unroll
-            for (int i = 0; i < NF; ++i)
-                if (j[i] >= 0) q.w[i][u] = Coef<F>::adj_once(m, e.z + j[i] - (j[i] > e.x ? 1 : 0));
+        for (int i = 0; i < NF; ++i) {
+            q.w[i][u] = F(0);
+            if (on && j[i] >= 0) q.w[i][u] = Coef<F>::adj_once(m, e.z + j[i] - (j[i] > e.x ? 1 : 0));
+        }
+    }
+}
+template <class F, int NF, int NR>
+__device__ __forceinline__ void add_rows(const RowPart<F, NF, NR>& q, F (&f)[NF]) {
+#pragma unroll
+    for (int u = 0; u < NR; ++u)
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            F g = f[i];
+            solo_add(&g, q.w[i][u], q.dz[u]);
+            f[i] = q.dz[u] != 0 ? g : f[i];
         }
 }
-template <class F, int NF>
-__device__ __forceinline__ void add_rows(const RowPart<F, NF>& q, const Commit* list, int c, int count, F (&f)[NF]) {
-#pragma unroll
-    for (int u = 0; u < kRows<F>; ++u)
-        if (c + u < count) {
-            const int dz = list[c + u].y;
-#pragma unroll
-            for (int i = 0; i < NF; ++i) solo_add(&f[i], q.w[i][u], dz);
-        }
-}
-// Every field outside of blocks b0 and b1, by threads t = 0..nt-1.
+// Every field outside of blocks b0 and b1, by threads t = 0..nt-1: four fields
+// (two for int64) with eight (four) rows each in flight per thread.  A pass is
+// one L2 round trip, about 1700 cycles when every SM reads rows: with two fields
+// at a time the 1000-variable case below took 6.8 ms instead of 6.4.
 template <class F, int MEM>
 __device__ __noinline__ void add_commits(const DevModel& m, F* cache_any, const Commit* list_any, int count, int b0,
                                          int b1, int t, int nt) {
+    constexpr int NF = Num<F>::is_float ? 4 : 2, NR = Num<F>::is_float ? 8 : 4;
     F* cache = in_shared<MEM>(cache_any);
     const Commit* list = in_shared<MEM>(list_any);
-    for (int j0 = t; j0 < m.n; j0 += 2 * nt) {
-        int j[2] = {j0, j0 + nt};
-        if ((j[0] >> 5) == b0 || (j[0] >> 5) == b1) j[0] = -1;
-        if (j[1] >= m.n || (j[1] >> 5) == b0 || (j[1] >> 5) == b1) j[1] = -1;
-        F f[2] = {F(0), F(0)};
+    const int n = m.n;
+    for (int j0 = t; j0 < n; j0 += NF * nt) {
+        int j[NF];
+        F f[NF];
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-            if (j[i] >= 0) f[i] = cache[j[i]];
-        for (int c = 0; c < count; c += kRows<F>) {
-            RowPart<F, 2> q;
-            load_rows<F, 2>(q, m, list, c, count, j);
-            add_rows<F, 2>(q, list, c, count, f);
+        for (int i = 0; i < NF; ++i) {
+            j[i] = j0 + i * nt;
+            if (j[i] >= n || (j[i] >> 5) == b0 || (j[i] >> 5) == b1) j[i] = -1;
+            f[i] = j[i] >= 0 ? cache[j[i]] : F(0);
+        }
+        for (int c = 0; c < count; c += NR) {
+            RowPart<F, NF, NR> q;
+            load_rows<F, NF, NR>(q, m, list, c, count, j);
+            add_rows<F, NF, NR>(q, f);
         }
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+        for (int i = 0; i < NF; ++i)
             if (j[i] >= 0) cache[j[i]] = f[i];
     }
 }
@@ -306,6 +327,43 @@ __device__ __forceinline__ void group_scatter(const DevModel& m, F* cache, const
 }
 
 // ------------------------------------------------------------------ one block
+// Block b's couplings, records and masks on their way into one of the two
+// staged places (asynchronous 16-byte copies, issued one block ahead: an
+// L1 prefetch of the same lines left every coupling row an L2 round trip, about
+// 600 cycles a round).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+template <int MEM>
+__device__ __forceinline__ void stage_block(const DevModel& m, uint8_t* place, int b, int lane, bool records) {
+    const int4* w = reinterpret_cast<const int4*>(m.blk_w + (size_t)b * 1024);
+    const int4* rec = reinterpret_cast<const int4*>(m.idx_rec + b * 32);
+    const int recs = records ? min(32, m.n - b * 32) : 0;
+    int4* dw = reinterpret_cast<int4*>(place);
+    int4* dr = reinterpret_cast<int4*>(place + 4096);
+    uint32_t* dm = reinterpret_cast<uint32_t*>(place + 4096 + 32 * sizeof(LevelRec));
+    bool shared = MEM == MEM_SHARED;
+    if constexpr (MEM == MEM_EITHER) shared = __isShared(place);
+    if (shared) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cp_async16(dw + 32 * i + lane, w + 32 * i + lane);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (32 * i + lane < 2 * recs) cp_async16(dr + 32 * i + lane, rec + 32 * i + lane);
+        if (lane < recs) cp_async4(dm + lane, m.blk_mask + b * 32 + lane);
+    } else {
+        for (int i = lane; i < 256; i += 32) dw[i] = __ldg(w + i);
+        for (int i = lane; i < 2 * recs; i += 32) dr[i] = __ldg(rec + i);
+        if (lane < recs) dm[lane] = __ldg(m.blk_mask + b * 32 + lane);
+    }
+}
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // A lane's variable: what its decisions need besides the field.
 template <class F>
 struct BlockLane {
@@ -321,11 +379,10 @@ struct BlockLane {
 };
 
 // Block b's records, random words and proposals: nothing here waits for the
-// changes of earlier blocks.  The next block's records and couplings are
-// prefetched into L1 (couplings: one 128-byte line per variable, two for int64).
+// changes of earlier blocks.
 template <class F, class Z, int RULE>
-__device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* zs, int b, int s, int r, float ratio,
-                                                   int lane) {
+__device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* zs, const int4* recs,
+                                                   const uint32_t* masks, int b, int s, int r, int lane) {
     const DevModel& m = a.m;
     BlockLane<F> q;
     q.k = b * 32 + lane;
@@ -333,18 +390,10 @@ __device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* 
     q.nbr = 0;
     q.zo = 0;
     if (q.k < m.n) {
-        const int4* p = reinterpret_cast<const int4*>(m.idx_rec + q.k);
-        x0 = __ldg(p);
-        x1 = __ldg(p + 1);
-        q.nbr = __ldg(m.blk_mask + q.k);
+        x0 = recs[2 * lane];
+        x1 = recs[2 * lane + 1];
+        q.nbr = masks[lane];
         q.zo = (uint32_t)zs[q.k];
-    }
-    const int kn = q.k + 32;
-    if (kn < m.n) {
-        prefetch_l1(m.idx_rec + kn);
-        prefetch_l1(m.blk_mask + kn);
-#pragma unroll
-        for (int o = 0; o < (int)sizeof(F) / 4; ++o) prefetch_l1(Coef<F>::blk(m) + (size_t)kn * 32 + 16 * o);
     }
     q.lo = x0.y;
     q.width = (uint32_t)x0.z;
@@ -358,7 +407,7 @@ __device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* 
     q.prop = q.z;
     q.opt = false;
     if (RULE != RULE_HEAT_BATH && q.width != 0u) {
-        if (RULE == RULE_OPT) q.opt = unit_open_right(q.x.x2) < ratio;
+        if (RULE == RULE_OPT) q.opt = unit_open_right(q.x.x2) < __ldg(a.ratio + s);
         if (!q.opt) {
             const uint32_t j = pick_below(q.x.x0, q.width);
             q.prop = (long long)q.lo + (long long)(j >= q.zo ? j + 1u : j);
@@ -370,13 +419,19 @@ __device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* 
 // Decides block b (warp-collective) from the lanes' fields; on return f holds
 // every change of the block, the list its commits.  Returns their number.
 template <class F, class Z, int RULE>
-__device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<F>& q, Z* zs, F& f, Commit* list, int b,
-                                            int s, int r, float beta, float temp, int lane, SweepAcc<F>& acc) {
+__device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<F>& q, const uint8_t* place, Z* zs, F& f,
+                                            Commit* list, int b, int s, int r, float beta, float temp, int lane,
+                                            SweepAcc<F>& acc) {
     constexpr unsigned full = 0xffffffffu;
     const DevModel& m = a.m;
-    const F* const blk = Coef<F>::blk(m) + (size_t)b * 1024 + lane;   // row p of the block: blk[32 p]
+    // row p of the block's couplings
+    const int* const blk = reinterpret_cast<const int*>(place) + lane;
+    auto coupling = [&](int p) -> F {
+        if constexpr (Num<F>::is_float) return __int_as_float(blk[32 * p]);
+        else return m.blk_i == nullptr ? (long long)blk[32 * p] : __ldg(m.blk_i + (size_t)b * 1024 + 32 * p + lane);
+    };
     const long long z = q.z;
-    long long v = z, prop = q.prop;
+    long long v = z;
     int count = 0;
     // heat bath: narrow ranges are decided by the lanes (rounds, like the other
     // rules) unless most of the last block changed; other ranges one variable
@@ -393,7 +448,7 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
         while (left) {
             const int p = __ffs(left) - 1;
             left &= left - 1u;
-            const F w = __ldg(blk + 32 * p);
+            const F w = coupling(p);
             VarView<F, KIND_QUIO> vv;
             vv.f = __shfl_sync(full, f, p);
             vv.d = __shfl_sync(full, q.d, p);
@@ -421,60 +476,93 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
             }
         }
     } else {
-        unsigned open = __ballot_sync(full, q.width != 0u);   // lanes still to be decided
+        // A round keeps to one path for all lanes and writes nothing: the list,
+        // the state and the energy follow when the block is decided.
+        unsigned open = __ballot_sync(full, q.width != 0u), changed = 0u;   // lanes still to be decided, changed
+        const bool chain = m.dense_rows != 0;
+        const float u = unit_open_right(q.x.x1);
+        // the proposal's share of dE = (v - z) (f + J_kk (v + z)) (quio_delta)
+        int dz = 0, dz_done = 0;
+        F dv = F(0), sv = F(0), de = F(0);
+        auto propose = [&](long long pv) {
+            dz = (int)(pv - z);
+            if constexpr (Num<F>::is_float) {
+                const float vf = __int2float_rn((int)pv), zf = __int2float_rn((int)z);
+                dv = vf - zf;
+                sv = vf + zf;
+            } else {
+                dv = pv - z;
+                sv = q.d * (pv + z);
+            }
+        };
+        propose(q.prop);
         while (open) {
-            F de = F(0);
-            bool chg = false;
-            if ((open >> lane) & 1u) {
-                VarView<F, KIND_QUIO> vv;
-                vv.f = f;
-                vv.d = q.d;
-                if constexpr (RULE == RULE_HEAT_BATH) {
-                    if (vv.linear()) prop = heat_bath_linear(Num<F>::to_f(f), q.lo, q.width, q.x.x0, beta);
-                    else if constexpr (Num<F>::is_float) {
-                        if (q.lo > -(1 << 22) && (long long)q.lo + (long long)q.width < (1 << 22))
-                            prop = heat_bath_quio_f32_small((float)f, (float)q.d, z, q.lo, q.width, q.x.x0, beta, temp);
-                        else
-                            prop = heat_bath_general<F, KIND_QUIO>(vv, z, q.lo, q.width, q.x.x0, beta);
-                    } else {
-                        prop = heat_bath_narrow(vv, z, q.lo, q.width, q.x.x0, beta, m.max_width);
-                    }
-                    chg = prop != z;
-                    if (chg) de = vv.delta(z, prop);
-                } else {
-                    if (RULE == RULE_OPT && q.opt)
-                        prop = opt_argmin<F, KIND_QUIO>(vv, z, q.lo, (long long)q.lo + (long long)q.width);
-                    de = quio_delta<F>(f, q.d, z, prop);
-                    chg = prop != z && metropolis_accept<F>(de, q.x.x1, beta);
+            const bool mine = (open >> lane) & 1u;
+            if constexpr (RULE == RULE_HEAT_BATH) {
+                if (mine) propose(heat_bath_lane<F>(f, q.d, (int)z, q.lo, q.width, q.x.x0, beta, temp, m.max_width));
+            } else if constexpr (RULE == RULE_OPT) {
+                if (mine && q.opt) {
+                    VarView<F, KIND_QUIO> vv;
+                    vv.f = f;
+                    vv.d = q.d;
+                    propose(opt_argmin<F, KIND_QUIO>(vv, z, q.lo, (long long)q.lo + (long long)q.width));
                 }
+            }
+            F dn;
+            if constexpr (Num<F>::is_float) dn = __fmul_rn(dv, fmaf(q.d, sv, f));
+            else dn = dv * (f + sv);
+            bool chg = mine & (dz != 0);
+            if (RULE != RULE_HEAT_BATH) {   // metropolis_accept without its branch
+                const float pr = expf(-(Num<F>::to_f(dn) * beta));
+                chg = chg & ((dn <= F(0)) | (u < pr));
             }
             const unsigned c = __ballot_sync(full, chg);
             if (!c) break;
-            // the first lane whose field one of the changes reaches decides again
-            const unsigned late = __ballot_sync(full, ((open >> lane) & 1u) && (q.nbr & c) != 0u);
-            const unsigned done = late ? (late & (0u - late)) - 1u : full;
-            unsigned com = c & done;
-            if ((com >> lane) & 1u) {
-                v = prop;
-                list[count + __popc(com & ((1u << lane) - 1u))] = make_int4(q.k, (int)(v - z), q.row, q.len);
-                zs[q.k] = (Z)(v - (long long)q.lo);
-                ++acc.changes;
-                if constexpr (!Num<F>::is_float) acc.e += de;
+            // the first lane whose field one of the changes reaches decides
+            // again; on a complete graph that is the next lane
+            unsigned done;
+            if (chain) {
+                const unsigned low = c & (0u - c);
+                done = low | (low - 1u);
+            } else {
+                const unsigned late = __ballot_sync(full, mine && (q.nbr & c) != 0u);
+                done = late ? (late & (0u - late)) - 1u : full;
             }
-            count += __popc(com);
-            const int dz = (int)(prop - z);
-            while (com) {
+            unsigned com = c & done;
+            changed |= com;
+            open &= ~done;
+            const bool now = (com >> lane) & 1u;
+            dz_done = now ? dz : dz_done;
+            de = now ? dn : de;
+            do {
                 const int p = __ffs(com) - 1;
                 com &= com - 1u;
-                const F w = __ldg(blk + 32 * p);
-                const int dp = __shfl_sync(full, dz, p);
-                if (lane != p) solo_add(&f, w, dp);
-                if constexpr (Num<F>::is_float) {   // summed in the visiting order, by one lane
-                    const float ep = __shfl_sync(full, (float)de, p);
-                    if (lane == 0) acc.de = __fadd_rn(acc.de, ep);
+                F g = f;
+                solo_add(&g, coupling(p), __shfl_sync(full, dz, p));
+                f = lane != p ? g : f;
+            } while (com);
+        }
+        count = __popc(changed);
+        v = z + dz_done;
+        if ((changed >> lane) & 1u) {
+            list[__popc(changed & ((1u << lane) - 1u))] = make_int4(q.k, dz_done, q.row, q.len);
+            zs[q.k] = (Z)(v - (long long)q.lo);
+            ++acc.changes;
+            if constexpr (!Num<F>::is_float) acc.e += de;
+        }
+        if constexpr (Num<F>::is_float) {   // summed in the visiting order, by one lane, four at a time
+            for (unsigned c = changed; c;) {
+                float ep[4];
+                bool on[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    on[i] = c != 0u;
+                    ep[i] = __shfl_sync(full, (float)de, __ffs(c | 0x80000000u) - 1);
+                    c &= c - 1u;
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc.de = on[i] && lane == 0 ? __fadd_rn(acc.de, ep[i]) : acc.de;
             }
-            open &= ~done;
         }
     }
     if constexpr (RULE == RULE_HEAT_BATH) acc.busy = count;
@@ -483,60 +571,106 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
     return count;
 }
 
+// Whether two warps take the blocks of a complete graph in turn: the one that
+// does not decide makes the next block's random words and proposals (they need
+// no field) and fetches its couplings, so that the deciding warp only adds the
+// last changes and runs its rounds.  Each warp has a staged place of its own.
+__device__ __forceinline__ bool block_pair(int tpr, int nb) { return tpr >= 128 && nb >= 2; }
+template <class F, class Z, int RULE, int MEM>
+__device__ __forceinline__ void prepare_block(const SweepArgs& a, const Z* zs, uint8_t* place, int b, int s, int r,
+                                              int lane, BlockLane<F>& q) {
+    if (s >= a.S) return;
+    stage_block<MEM>(a.m, place, b, lane, false);
+    q = block_lane<F, Z, RULE>(a, zs, reinterpret_cast<const int4*>(a.m.idx_rec + b * 32), a.m.blk_mask + b * 32, b, s,
+                               r, lane);
+}
+
 // ------------------------------------------------------------------ one sweep
 // Sweep s of replica r in blocks.  `flush`: the caller needs the state at the
 // end of this sweep (a refresh, a trace, the outputs), so the last block's
 // changes are applied before returning; otherwise they wait for the next sweep.
 //
-// Complete graphs: while warp 0 decides block b, the other warps add the changes
-// of block b - 1 to every field outside of blocks b - 1 and b (each field by one
-// thread, its rows eight loads deep); warp 0 adds them to block b's fields
-// itself when it starts on them.  One barrier per block.
+// Complete graphs: while one warp decides block b, the others add the changes of
+// block b - 1 to every field outside of blocks b - 1 and b (each field by one
+// thread); the deciding warp adds them to block b's fields itself when it starts
+// on them.  One barrier per block.
 // Other graphs: warp 0 decides, then the group scatters the block's rows by
 // their columns; short rows are scattered by warp 0 without waking the others.
 // Float models whose every level holds one variable keep the order of the
 // additions (one commit at a time).
 template <class F, class Z, int RULE, int MEM>
-__device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache, int* ctl, Commit* lists, int bar_id,
-                                            int t, int tpr, int r, int s, bool flush, SweepAcc<F>& acc) {
+__device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache, int* ctl, Commit* lists, uint8_t* stage,
+                                            int bar_id, int t, int tpr, int r, int s, bool flush, SweepAcc<F>& acc,
+                                            BlockLane<F>& q) {
     const DevModel& m = a.m;
     const int lane = t & 31;
     const float beta = __ldg(a.beta + s);
     const float temp = 1.f / beta;
-    const float ratio = __ldg(a.ratio + s);
     const int nb = (m.n + 31) >> 5;
+    // warp 0, at the start of block b: its staged place, with the next block's
+    // copies issued (a model of one or two blocks stays staged), and its lanes
+    auto begin = [&](int b) -> const uint8_t* {
+        const uint8_t* place = stage + (nb > 2 ? (acc.turn & 1) : b) * kBlockStage;
+        if (nb > 2) {
+            stage_wait();
+            __syncwarp();   // every lane's copies of block b are there; block b - 1's place is free
+            ++acc.turn;
+            stage_block<MEM>(m, stage + (acc.turn & 1) * kBlockStage, b + 1 < nb ? b + 1 : 0, lane, true);
+        }
+        q = block_lane<F, Z, RULE>(a, zs, reinterpret_cast<const int4*>(place + 4096),
+                                   reinterpret_cast<const uint32_t*>(place + 4096 + 32 * sizeof(LevelRec)), b, s, r, lane);
+        return place;
+    };
     if (m.dense_rows) {
+        const bool pair = block_pair(tpr, nb);
+        const int first = pair ? 64 : (tpr > 32 ? 32 : 0);   // first thread that only adds rows
+        float* run = reinterpret_cast<float*>(ctl) + 8 + (s & 1);   // the sweep's energy change so far (float models)
         for (int b = 0; b < nb; ++b) {
             const Commit* prev = lists + 32 * (acc.par ^ 1);
             const int np = acc.last >= 0 ? ctl[acc.par ^ 1] : 0;
-            if (t < 32) {
+            if (pair ? (t >> 5) == acc.par : t < 32) {
                 const int k = b * 32 + lane;
                 const int ahead = acc.last != b ? np : 0;
                 F f[1] = {k < m.n ? cache[k] : F(0)};
-                // the first rows of the last block's changes are on their way
-                // while this block's random words are made
                 const int j[1] = {k < m.n ? k : -1};
-                RowPart<F, 1> rows;
-                load_rows<F, 1>(rows, m, prev, 0, ahead, j);
-                const BlockLane<F> q = block_lane<F, Z, RULE>(a, zs, b, s, r, ratio, lane);
-                add_rows<F, 1>(rows, prev, 0, ahead, f);
-                for (int c = kRows<F>; c < ahead; c += kRows<F>) {
-                    load_rows<F, 1>(rows, m, prev, c, ahead, j);
-                    add_rows<F, 1>(rows, prev, c, ahead, f);
+                constexpr int NR = 8;
+                RowPart<F, 1, NR> ra, rb;
+                load_rows<F, 1, NR>(ra, m, prev, 0, ahead, j);
+                if (ahead > NR) load_rows<F, 1, NR>(rb, m, prev, NR, ahead, j);
+                const uint8_t* place = stage + acc.par * kBlockStage;
+                if (pair) {
+                    stage_wait();
+                    __syncwarp();
+                    if (lane == 0) acc.de = b > 0 ? *run : 0.f;
+                } else {
+                    place = begin(b);
                 }
-                const int cnt = decide_block<F, Z, RULE>(a, q, zs, f[0], lists + 32 * acc.par, b, s, r, beta, temp,
-                                                         lane, acc);
+                add_rows<F, 1, NR>(ra, f);
+                if (ahead > NR) add_rows<F, 1, NR>(rb, f);
+                for (int c = 2 * NR; c < ahead; c += NR) {
+                    load_rows<F, 1, NR>(ra, m, prev, c, ahead, j);
+                    add_rows<F, 1, NR>(ra, f);
+                }
+                const int cnt = decide_block<F, Z, RULE>(a, q, place, zs, f[0], lists + 32 * acc.par, b, s, r, beta,
+                                                         temp, lane, acc);
                 if (k < m.n) cache[k] = f[0];
-                if (lane == 0) ctl[acc.par] = cnt;
+                if (lane == 0) {
+                    ctl[acc.par] = cnt;
+                    if (pair) {
+                        *run = acc.de;
+                        acc.de = 0.f;
+                    }
+                }
+            } else if (pair && t < 64) {
+                prepare_block<F, Z, RULE, MEM>(a, zs, stage + (acc.par ^ 1) * kBlockStage, b + 1 < nb ? b + 1 : 0,
+                                               b + 1 < nb ? s : s + 1, r, lane, q);
             }
-            if (np > 0 && (t >= 32 || tpr == 32)) {
-                const int skip = tpr > 32 ? 32 : 0;
-                add_commits<F, MEM>(m, cache, prev, np, acc.last, b, t - skip, tpr - skip);
-            }
+            if (np > 0 && t >= first) add_commits<F, MEM>(m, cache, prev, np, acc.last, b, t - first, tpr - first);
             named_bar(bar_id, tpr);
             acc.par ^= 1;
             acc.last = b;
         }
+        if (pair && t == 0) acc.de = *run;   // (read before the place's next use, two sweeps on)
         if (flush) {
             add_commits<F, MEM>(m, cache, lists + 32 * (acc.par ^ 1), ctl[acc.par ^ 1], acc.last, acc.last, t, tpr);
             named_bar(bar_id, tpr);
@@ -550,8 +684,8 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
             for (int b = 0; b < nb; ++b) {
                 const int k = b * 32 + lane;
                 F f = k < m.n ? cache[k] : F(0);
-                const BlockLane<F> q = block_lane<F, Z, RULE>(a, zs, b, s, r, ratio, lane);
-                const int cnt = decide_block<F, Z, RULE>(a, q, zs, f, lists, b, s, r, beta, temp, lane, acc);
+                const uint8_t* place = begin(b);
+                const int cnt = decide_block<F, Z, RULE>(a, q, place, zs, f, lists, b, s, r, beta, temp, lane, acc);
                 if (k < m.n) cache[k] = f;
                 __syncwarp();
                 if (cnt == 0 || nb == 1) continue;
@@ -599,13 +733,27 @@ __device__ __forceinline__ void block_run(const SweepArgs& a, uint8_t* base, int
     int* ctl = reinterpret_cast<int*>(base + a.off_ctl);
     Commit* lists = reinterpret_cast<Commit*>(base + a.off_list);   // two lists of 32
     typename Num<F>::Acc* red = reinterpret_cast<typename Num<F>::Acc*>(base + a.off_red);
+    uint8_t* stage = base + a.off_blk;
+    const int nb = (a.m.n + 31) >> 5;
+    BlockLane<F> q{};
+    if (t < 32) {   // the first block, or all of one or two
+        if (a.m.dense_rows && block_pair(tpr, nb)) {
+            prepare_block<F, Z, RULE, MEM>(a, zs, stage, 0, s0, r, t, q);
+        } else {
+            stage_block<MEM>(a.m, stage, 0, t, true);
+            if (nb == 2) stage_block<MEM>(a.m, stage + kBlockStage, 1, t, true);
+            stage_wait();
+            __syncwarp();
+        }
+    }
     for (int s = s0; s < s1; ++s) {
         const bool flush = s + 1 == s1 || a.energy_trace != nullptr || a.best_states != nullptr ||
                            (Num<F>::is_float && a.refresh_interval > 0 && (s + 1) % a.refresh_interval == 0);
-        block_sweep<F, Z, RULE, MEM>(a, zs, cache, ctl, lists, bar_id, t, tpr, r, s, flush, acc);
-        end_of_sweep<F, Z, KIND_QUIO>(a, zs, cache, red, t, tpr, bar_id, r, s, s == s0 && fresh, acc.e, acc.de,
+        block_sweep<F, Z, RULE, MEM>(a, zs, cache, ctl, lists, stage, bar_id, t, tpr, r, s, flush, acc, q);
+        end_of_sweep<F, Z, KIND_QUIO, MEM, true>(a, zs, cache, red, t, tpr, bar_id, r, s, s == s0 && fresh, acc.e, acc.de,
                                       acc.drift);
     }
+    stage_wait();   // no copy is in flight when the region is given up
 }
 
 }  // namespace dev
