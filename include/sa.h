@@ -152,7 +152,7 @@ typedef struct {
 /* Run flags */
 #define SA_FLAG_STATE_IN_GLOBAL 0x1   /* keep per-replica state in global memory even if it fits on chip */
 #define SA_FLAG_NO_TIME_SLICING 0x2   /* run more replicas than fit at once as plain waves (see sa_run) */
-#define SA_FLAG_NO_SPECULATION  0x4   /* decide single-variable levels one at a time (see sa_run) */
+#define SA_FLAG_NO_SPECULATION  0x4   /* sweep level by level, not in blocks (see sa_run) */
 
 typedef struct {
     int32_t rule;                 /* sa_rule                                              */
@@ -213,16 +213,15 @@ typedef struct {
  * concurrently when they form a dependency level; this reproduces the
  * sequential trajectory exactly for integer models.
  *
- * Speculative windows (QUIO): a run of levels that hold one variable each
- * (every level of a complete graph) is decided by the lanes of one warp, up
- * to 32 levels at once.  The decisions before the first one that changes its
- * variable saw the same state as in the sequential order, and so did that
- * one; its neighbours' fields are then updated and the next window starts
- * after it.  States, energies, counts and traces are those of the
- * level-by-level order, bit for bit (float models included).  Float heat bath,
- * and heat bath where a variable's range makes the kernel decide it with a
- * whole warp, keep the level-by-level order.  SA_FLAG_NO_SPECULATION disables
- * the windows.
+ * Blocked sweeps (QUIO): models whose levels are narrow (up to 16 variables on
+ * average, up to 3 for the heat bath; every level of a complete graph holds
+ * one) are swept in blocks of 32 consecutive variables, decided by one warp at
+ * once.  A decision is kept when no earlier variable of the block that shares a
+ * term with it changes in the same round; the others are made again with the
+ * changes in their fields.  States, counts and traces are those of the
+ * level-by-level order, bit for bit (float models included where every level
+ * holds one variable, and energies too at the same thread count).
+ * SA_FLAG_NO_SPECULATION keeps the level-by-level order.
  *
  * Time slicing: when the replicas' state stays in shared memory but more
  * replicas are requested than thread groups fit on the GPU at once, and the

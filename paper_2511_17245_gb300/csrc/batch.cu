@@ -106,6 +106,15 @@ sa_status apply_shape(sa_batch* b, int tpr, int rpc_req) {
                                             2048 / (rpc * tpr)));
     else per_sm = std::max(1, 2048 / (rpc * tpr));
     per_sm = std::min(per_sm, std::max(1, 65536 / (rpc * tpr * 128)));   // registers: up to 128 per thread
+    // blocked instances stage their blocks behind the regions where there is room
+    bool any_blocked = false;
+    for (const auto& a : b->h_insts) any_blocked = any_blocked || a.blocked;
+    if (smem && any_blocked && (size_t)rpc * (slot + 2 * sa::kBlockStage) <= (size_t)std::max(0, smem_max) &&
+        std::max(1, (int)((size_t)sa::sweep_max_shared_optin() / ((size_t)rpc * (slot + 2 * sa::kBlockStage) + 8192))) >= per_sm) {
+        for (auto& a : b->h_insts)
+            if (a.blocked) a.off_blk = (int32_t)slot;
+        slot += 2 * sa::kBlockStage;
+    }
     int blocks = sms * per_sm;
     const int need = (int)((b->h_units.size() + rpc - 1) / rpc);
     blocks = std::max(1, std::min(blocks, need));

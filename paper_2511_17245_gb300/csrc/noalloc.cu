@@ -106,13 +106,18 @@ extern "C" sa_status sa_run_noalloc(const sa_model* M, const sa_run_params* p, i
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sa::RunPlan plan{};
-    if (const char* err = sa::plan_run(sa::plan_model(mv), p->rule, !(p->flags & SA_FLAG_NO_SPECULATION), R,
-                                       p->threads_per_replica, p->replicas_per_block,
-                                       (p->flags & SA_FLAG_STATE_IN_GLOBAL) != 0, sms,
-                                       sa::sweep_max_shared_optin(), &plan))
-        return fail(SA_ERR_INVALID, err);
+    auto make_plan = [&](int32_t threads) {
+        return sa::plan_run(sa::plan_model(mv), p->rule, !(p->flags & SA_FLAG_NO_SPECULATION), R, threads,
+                            p->replicas_per_block, (p->flags & SA_FLAG_STATE_IN_GLOBAL) != 0, sms,
+                            sa::sweep_max_shared_optin(), &plan);
+    };
+    if (const char* err = make_plan(p->threads_per_replica)) return fail(SA_ERR_INVALID, err);
+    auto slab = [&]() { return plan.in_global ? (size_t)R * (size_t)plan.rep_bytes : (size_t)0; };
+    // each warp of a replica adds a few bytes to its region: the smallest shape
+    // decides whether the slab fits
+    if (p->threads_per_replica <= 0 && tab_bytes + slab() > (size_t)SA_NOALLOC_SCRATCH_BYTES) make_plan(plan.hb_tpr);
     const bool in_global = plan.in_global != 0;
-    const size_t slab_bytes = in_global ? (size_t)R * (size_t)plan.rep_bytes : 0;
+    const size_t slab_bytes = slab();
     if (tab_bytes + slab_bytes > (size_t)SA_NOALLOC_SCRATCH_BYTES)
         return fail(SA_ERR_UNSUPPORTED, "replica state does not fit on chip and " + std::to_string(R) +
                                             " replicas exceed the fixed scratch of sa_run_noalloc (" +

@@ -128,7 +128,7 @@ struct SweepArgs {
     uint8_t* gstate;            // per-replica state slabs when not on chip
     int64_t rep_bytes;          // bytes of one replica's state region
     int32_t off_z, off_cache, off_ctl, off_list, off_red;
-    int32_t off_blk;            // blocked sweeps: two staged blocks (kBlockStage bytes each)
+    int32_t off_blk;            // blocked sweeps: two staged blocks (kBlockStage bytes each; -1: not staged)
     int32_t off_lvl;            // level boundaries staged in the replica region (-1: read from the model)
     int32_t blocked;            // sweep in blocks of 32 variables (the model has idx_rec)
     int32_t hb_tpr;             // threads per replica that decide the form of heat-bath sums (hb_warp_mode)
@@ -342,8 +342,8 @@ inline int64_t plan_round16(int64_t x) { return (x + 15) / 16 * 16; }
 // each), the cache (int64 or fp32), the control words (three list counters or
 // the commit counts and commands of a blocked sweep), the cooperative update
 // list or a blocked sweep's two commit lists, the reduction scratch (one 8-byte word
-// per warp), when it takes at most 16 KB the level boundary table, and for models
-// of blocked sweeps two staged blocks.
+// per warp) and, when it takes at most 16 KB, the level boundary table.  (The
+// staged blocks of a blocked sweep come after it where they fit, see plan_run.)
 // `zbytes` may exceed the model's own (a batch uses its widest).  QUIO rows are
 // cheap per entry (one atomic) and go inline up to 64 links; HUIO incidences
 // cost a term product each and go inline up to 8.
@@ -362,8 +362,8 @@ inline int64_t plan_layout(const PlanModel& m, int zbytes, int tpr, RunPlan* p) 
     const int64_t off_lvl = plan_round16(p->off_red + (int64_t)(tpr / 32) * 8);
     const bool lvl_on_chip = lvl_bytes <= 16384;
     p->off_lvl = lvl_on_chip ? (int32_t)off_lvl : -1;
-    p->off_blk = (int32_t)plan_round16(off_lvl + (lvl_on_chip ? lvl_bytes : 0));
-    p->rep_bytes = p->off_blk + (m.block_model ? 2 * kBlockStage : 0);
+    p->off_blk = -1;
+    p->rep_bytes = plan_round16(off_lvl + (lvl_on_chip ? lvl_bytes : 0));
     return p->rep_bytes;
 }
 
@@ -428,6 +428,13 @@ inline const char* plan_run(const PlanModel& m, int rule, bool allow_blocks, int
     }
     p->blocked = blocked && allow_blocks ? 1 : 0;
     p->hb_tpr = hb_tpr;
+    // staged blocks only where there is room: they never change which shapes and
+    // placements are possible
+    if (p->blocked && !p->in_global && (p->rep_bytes + 2 * kBlockStage) * p->rpc + 1024 <= smem_max) {
+        p->off_blk = (int32_t)p->rep_bytes;
+        p->rep_bytes += 2 * kBlockStage;
+        p->shared_bytes = p->rep_bytes * p->rpc;
+    }
     return nullptr;
 }
 

@@ -186,6 +186,7 @@ bool admit(sa_server* s, Request* r, int slot) {
     pl.rpc = s->args.rpc;
     pl.blocked = sa::plan_blocked(sa::plan_model(v), p.rule, !(p.flags & SA_FLAG_NO_SPECULATION));
     pl.hb_tpr = s->args.tpr;
+    if (pl.blocked && !r->slab && pl.rep_bytes + 2 * sa::kBlockStage <= s->args.slot_bytes) pl.off_blk = (int32_t)pl.rep_bytes;
     sa::plan_apply(pl, a);
     sa::ServeReq& q = s->h_reqs[slot];
     q.args = a;

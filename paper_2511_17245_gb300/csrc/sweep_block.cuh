@@ -381,8 +381,8 @@ struct BlockLane {
 // Block b's records, random words and proposals: nothing here waits for the
 // changes of earlier blocks.
 template <class F, class Z, int RULE>
-__device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* zs, const int4* recs,
-                                                   const uint32_t* masks, int b, int s, int r, int lane) {
+__device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* zs, const uint8_t* place, bool staged,
+                                                   int b, int s, int r, int lane) {
     const DevModel& m = a.m;
     BlockLane<F> q;
     q.k = b * 32 + lane;
@@ -390,9 +390,17 @@ __device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* 
     q.nbr = 0;
     q.zo = 0;
     if (q.k < m.n) {
-        x0 = recs[2 * lane];
-        x1 = recs[2 * lane + 1];
-        q.nbr = masks[lane];
+        if (staged) {
+            const int4* p = reinterpret_cast<const int4*>(place + 4096) + 2 * lane;
+            x0 = p[0];
+            x1 = p[1];
+            q.nbr = reinterpret_cast<const uint32_t*>(place + 4096 + 32 * sizeof(LevelRec))[lane];
+        } else {
+            const int4* p = reinterpret_cast<const int4*>(m.idx_rec + q.k);
+            x0 = __ldg(p);
+            x1 = __ldg(p + 1);
+            q.nbr = __ldg(m.blk_mask + q.k);
+        }
         q.zo = (uint32_t)zs[q.k];
     }
     q.lo = x0.y;
@@ -426,9 +434,12 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
     const DevModel& m = a.m;
     // row p of the block's couplings
     const int* const blk = reinterpret_cast<const int*>(place) + lane;
+    const bool staged = a.off_blk >= 0;
     auto coupling = [&](int p) -> F {
-        if constexpr (Num<F>::is_float) return __int_as_float(blk[32 * p]);
-        else return m.blk_i == nullptr ? (long long)blk[32 * p] : __ldg(m.blk_i + (size_t)b * 1024 + 32 * p + lane);
+        const size_t at = (size_t)b * 1024 + 32 * p + lane;
+        const int w = staged ? blk[32 * p] : __ldg(m.blk_w + at);
+        if constexpr (Num<F>::is_float) return __int_as_float(w);
+        else return m.blk_i == nullptr ? (long long)w : (long long)__ldg(m.blk_i + at);
     };
     const long long z = q.z;
     long long v = z;
@@ -580,9 +591,8 @@ template <class F, class Z, int RULE, int MEM>
 __device__ __forceinline__ void prepare_block(const SweepArgs& a, const Z* zs, uint8_t* place, int b, int s, int r,
                                               int lane, BlockLane<F>& q) {
     if (s >= a.S) return;
-    stage_block<MEM>(a.m, place, b, lane, false);
-    q = block_lane<F, Z, RULE>(a, zs, reinterpret_cast<const int4*>(a.m.idx_rec + b * 32), a.m.blk_mask + b * 32, b, s,
-                               r, lane);
+    if (a.off_blk >= 0) stage_block<MEM>(a.m, place, b, lane, false);
+    q = block_lane<F, Z, RULE>(a, zs, place, false, b, s, r, lane);
 }
 
 // ------------------------------------------------------------------ one sweep
@@ -610,15 +620,15 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
     // warp 0, at the start of block b: its staged place, with the next block's
     // copies issued (a model of one or two blocks stays staged), and its lanes
     auto begin = [&](int b) -> const uint8_t* {
+        const bool staged = a.off_blk >= 0;
         const uint8_t* place = stage + (nb > 2 ? (acc.turn & 1) : b) * kBlockStage;
-        if (nb > 2) {
+        if (staged && nb > 2) {
             stage_wait();
             __syncwarp();   // every lane's copies of block b are there; block b - 1's place is free
             ++acc.turn;
             stage_block<MEM>(m, stage + (acc.turn & 1) * kBlockStage, b + 1 < nb ? b + 1 : 0, lane, true);
         }
-        q = block_lane<F, Z, RULE>(a, zs, reinterpret_cast<const int4*>(place + 4096),
-                                   reinterpret_cast<const uint32_t*>(place + 4096 + 32 * sizeof(LevelRec)), b, s, r, lane);
+        q = block_lane<F, Z, RULE>(a, zs, place, staged, b, s, r, lane);
         return place;
     };
     if (m.dense_rows) {
@@ -733,13 +743,13 @@ __device__ __forceinline__ void block_run(const SweepArgs& a, uint8_t* base, int
     int* ctl = reinterpret_cast<int*>(base + a.off_ctl);
     Commit* lists = reinterpret_cast<Commit*>(base + a.off_list);   // two lists of 32
     typename Num<F>::Acc* red = reinterpret_cast<typename Num<F>::Acc*>(base + a.off_red);
-    uint8_t* stage = base + a.off_blk;
+    uint8_t* stage = base + (a.off_blk >= 0 ? a.off_blk : 0);   // (not touched where blocks are not staged)
     const int nb = (a.m.n + 31) >> 5;
     BlockLane<F> q{};
     if (t < 32) {   // the first block, or all of one or two
         if (a.m.dense_rows && block_pair(tpr, nb)) {
             prepare_block<F, Z, RULE, MEM>(a, zs, stage, 0, s0, r, t, q);
-        } else {
+        } else if (a.off_blk >= 0) {
             stage_block<MEM>(a.m, stage, 0, t, true);
             if (nb == 2) stage_block<MEM>(a.m, stage + kBlockStage, 1, t, true);
             stage_wait();

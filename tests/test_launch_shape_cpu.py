@@ -141,3 +141,30 @@ def test_time_sliced_tasks_cover_every_sweep_once(tmp_path, R, S, P):
     assert makespan <= R * per_replica / P + 2 * max_chunk + 1e-9
     waves = -(-R // P)
     assert makespan <= waves * per_replica + 1e-9
+
+
+@pytest.mark.parametrize("n,levels,dense,links,R,rule,want", [
+    (1501, 36, 0, 16, 512, "RULE_METROPOLIS", (96, 32, 0)),    # level by level: twice the mean width
+    (10000, 43, 0, 16, 1024, "RULE_METROPOLIS", (128, 128, 0)),  # four replicas of 51 KB fill the block: 128 threads each
+    (1000, 1000, 1, 999, 152, "RULE_METROPOLIS", (384, 256, 1)),  # complete graph: 3 n / 8 threads
+    (32, 32, 1, 31, 64, "RULE_HEAT_BATH", (32, 32, 1)),        # one block: one warp
+    (300, 60, 0, 40, 64, "RULE_METROPOLIS", (192, 32, 1)),     # narrow levels: blocks
+    (300, 60, 0, 40, 64, "RULE_HEAT_BATH", (32, 32, 0)),       # (the heat bath keeps levels wider than 3)
+])
+def test_plan_run_threads(tmp_path, n, levels, dense, links, R, rule, want):
+    """Thread count, heat-bath form's thread count and sweep form of a run; a
+    caller's thread count is kept."""
+    body = f"""
+  sa::PlanModel m{{{n}, {levels}, sa::KIND_QUIO, 1, 1, {links}, {n}, sa::plan_block_model({n}, {levels}), {dense}, {links}}};
+  sa::RunPlan p{{}};
+  sa::plan_run(m, sa::{rule}, true, {R}, 0, 0, false, 152, 232448, &p);
+  std::printf("%d %d %d\\n", p.tpr, p.hb_tpr, p.blocked);
+  sa::plan_run(m, sa::{rule}, false, {R}, 0, 0, false, 152, 232448, &p);
+  std::printf("%d %d\\n", p.tpr, p.blocked);
+  sa::plan_run(m, sa::{rule}, true, {R}, 64, 0, false, 152, 232448, &p);
+  std::printf("%d %d\\n", p.tpr, p.hb_tpr);
+"""
+    out = [int(x) for x in _compile_and_run(tmp_path, body)]
+    assert tuple(out[:3]) == want
+    assert out[3] == want[0] and out[4] == 0     # the level order runs with the same threads
+    assert out[5:] == [64, 64]
