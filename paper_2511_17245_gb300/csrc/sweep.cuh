@@ -606,15 +606,13 @@ __device__ long long heat_bath_general(const VarView<F, KIND>& vv, long long z, 
 // heat_bath_general of an integer QUIO variable with at most 32 values, one
 // lane, bit for bit the same pick: the one block of values is always kept, dE
 // walks up by exact differences, and the running sums of the first pass, which
-// the second pass would form again, stay in registers.  Sixteen values take
-// about a quarter of the time of the three loops.
-__device__ __forceinline__ long long heat_bath_narrow(const VarView<long long, KIND_QUIO>& vv, long long z,
-                                                      long long lo, uint32_t width, uint32_t xu, float beta,
-                                                      uint32_t max_width) {
-    long long mn = quio_interval_min<long long>(vv, z, lo, lo + (long long)width);
-    mn = mn < 0 ? mn : 0;
-    long long de = vv.delta(z, lo) - mn;
-    long long step = vv.f + vv.d * (2 * lo + 1);   // dE(v + 1) - dE(v) at v = lo
+// the second pass would form again, stay in registers.  Groups of eight values
+// up to the model's widest range, and selects instead of branches: what bounds
+// it is the chain of compensated additions, about 24 cycles a value.
+template <class T>
+__device__ __forceinline__ int narrow_pick(T de, T step, T dd, uint32_t width, uint32_t xu, float beta,
+                                           uint32_t max_width) {
+    // de, step: dE - dE_min at the first value and its first difference
     float run[32];
     float sum = 0.f, comp = 0.f;
 #pragma unroll
@@ -622,18 +620,24 @@ __device__ __forceinline__ long long heat_bath_narrow(const VarView<long long, K
 #pragma unroll
         for (int j = 0; j < 8; ++j) run[8 * g + j] = 0.f;
         if (8u * g <= max_width) {   // the same for every lane
+            float w[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                if ((uint32_t)(8 * g + j) <= width) {
-                    const float w = expf(-(Num<long long>::to_f(de) * beta));
-                    const float y = w - comp;
-                    const float t = sum + y;
-                    comp = (t - sum) - y;
-                    sum = t;
-                    run[8 * g + j] = sum;
-                }
+                float e;
+                if constexpr (sizeof(T) == 4) e = __int2float_rn(de);
+                else e = Num<long long>::to_f(de);
+                w[j] = expf(-(e * beta));
                 de += step;
-                step += 2 * vv.d;
+                step += dd;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const bool in = (uint32_t)(8 * g + j) <= width;
+                const float y = w[j] - comp;
+                const float t = sum + y;
+                comp = in ? (t - sum) - y : comp;
+                sum = in ? t : sum;
+                run[8 * g + j] = in ? t : 0.f;
             }
         }
     }
@@ -642,7 +646,36 @@ __device__ __forceinline__ long long heat_bath_narrow(const VarView<long long, K
 #pragma unroll
     for (int i = 31; i >= 0; --i)
         if (run[i] >= thr) pick = i;   // (thr > 0: a value past the range holds 0)
-    return lo + (long long)pick;
+    return pick;
+}
+
+__device__ __forceinline__ long long heat_bath_narrow(const VarView<long long, KIND_QUIO>& vv, long long z,
+                                                      long long lo, uint32_t width, uint32_t xu, float beta,
+                                                      uint32_t max_width) {
+    // small numbers: every dE of the range is below 32 (2^23 + 2^10 2^13) < 2^30,
+    // and all of it is 32-bit arithmetic; the minimum (0, at z, included) comes
+    // from the values themselves instead of a division
+    if (vv.f < (1 << 23) && vv.f > -(1 << 23) && vv.d < (1 << 10) && vv.d > -(1 << 10) && lo > -(1 << 12) &&
+        lo + (long long)width < (1 << 12)) {
+        const int f = (int)vv.f, d = (int)vv.d, l = (int)lo, zi = (int)z;
+        const int de0 = (l - zi) * (f + d * (l + zi)), step0 = f + d * (2 * l + 1);
+        int mn = 0, e = de0, st = step0;
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+            if (8u * g <= max_width) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    mn = (uint32_t)(8 * g + j) <= width ? min(mn, e) : mn;
+                    e += st;
+                    st += 2 * d;
+                }
+            }
+        return lo + (long long)narrow_pick<int>(de0 - mn, step0, 2 * d, width, xu, beta, max_width);
+    }
+    long long mn = quio_interval_min<long long>(vv, z, lo, lo + (long long)width);
+    mn = mn < 0 ? mn : 0;
+    return lo + (long long)narrow_pick<long long>(vv.delta(z, lo) - mn, vv.f + vv.d * (2 * lo + 1), 2 * vv.d, width, xu,
+                                                  beta, max_width);
 }
 
 // ------------------------------------------------------------------ warp-parallel heat bath
