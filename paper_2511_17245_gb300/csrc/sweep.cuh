@@ -1775,11 +1775,6 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
                                 Num<F>::is_float && KIND == KIND_QUIO && m.max_width < 256u);
         return false;
     };
-    // prefetch into L1 the records this thread will read in level L
-    auto prefetch_level = [&](int L) {
-        const int b0 = lvl_at(L), b1 = lvl_at(L + 1);
-        for (int i = b0 + t; i < b1; i += tpr) prefetch_l1(m.lvl_rec + i);
-    };
     if constexpr (BLK) {
         SweepAcc<F> io{eacc, changes, 0.f, drift, 0, 0, 0, -1};
         block_run<F, Z, RULE, MEM>(a, base, bar_id, t, r, s0, s1, restore == nullptr, io);
@@ -1787,19 +1782,24 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
         changes = io.changes;
         drift = io.drift;
     } else {
-    prefetch_level(0);
+    // Level boundaries are carried from level to level, and rounds are counted
+    // without a division: the start of a level took a warp 650 cycles before it
+    // looked at its first variable.
+    const int first_b = lvl_at(0), first_e = lvl_at(1);
     for (int s = s0; s < s1; ++s) {
         const float beta = __ldg(a.beta + s);
         const float temp = 1.f / beta;
         const float ratio = __ldg(a.ratio + s);
+        int lb = first_b, le = first_e;
         for (int L = 0; L < m.n_levels; ++L) {
             int* cnt_now = ctl + gl3;
             if (t == 0) ctl[gl3 == 2 ? 0 : gl3 + 1] = 0;
-            const int lb = lvl_at(L), le = lvl_at(L + 1);
             const bool wmode = wide_level(le - lb);
-            // the next level (the first level of the next sweep after the last)
-            if (L + 1 < m.n_levels) prefetch_level(L + 1);
-            else if (s + 1 < a.S) prefetch_level(0);
+            // prefetch into L1 the records this thread will read in the next level
+            // (the first level of the next sweep after the last)
+            const bool more = L + 1 < m.n_levels;
+            const int nb = more ? le : first_b, ne = more ? lvl_at(L + 2) : first_e;
+            for (int i = nb + t; i < ne; i += tpr) prefetch_l1(m.lvl_rec + i);
             // every thread of a warp runs the same number of rounds, so that the
             // warp can share the neighbour updates of its accepting lanes; heat
             // bath over wide ranges or narrow levels gives each variable a warp
@@ -1807,9 +1807,8 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
             const bool solo = le - lb == 1;
             const int per_round = wmode ? (tpr >> 5) : tpr;
             const int slot_i = wmode ? (t >> 5) : t;
-            const int rounds = (le - lb + per_round - 1) / per_round;
-            for (int rd = 0; rd < rounds; ++rd) {
-                const int i = lb + slot_i + rd * per_round;
+            for (int i0 = lb; i0 < le; i0 += per_round) {
+                const int i = i0 + slot_i;
                 bool coop = false;
                 int rb = 0, rl = 0;
                 long long rdz = 0;
@@ -1891,6 +1890,8 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
                 named_bar(bar_id, tpr);
             }
             gl3 = gl3 == 2 ? 0 : gl3 + 1;
+            lb = nb;
+            le = ne;
         }
         end_of_sweep<F, Z, KIND, MEM, BLK>(a, zs, cache, red, t, tpr, bar_id, r, s, s == s0 && restore == nullptr, eacc, dacc,
                                  drift);

@@ -36,10 +36,12 @@ struct SweepAcc {
 };
 
 // Heat bath over narrow ranges: a round of lane decisions settles 1 / p
-// variables when a share p of them changes and costs about 750 cycles (16
-// values), deciding them in turn about 550 each; above this many changes in the
-// last block they go in turn (the results are the same).
-constexpr int kBusyBlock = 22;
+// variables when a share p of them changes and costs about 2700 cycles (16
+// values: one warp issues an instruction every four to five cycles, and the
+// lanes' loops have some 500); in turn, with a variable's values spread over the
+// lanes, it is about 600 a variable.  Above this many changes in the last block
+// they go in turn (the results are the same).
+constexpr int kBusyBlock = 6;
 
 // A change of the block: {variable, z_new - z_old, first entry and length of its row}.
 using Commit = int4;
@@ -152,6 +154,44 @@ __device__ __forceinline__ long long heat_bath_small_warp(float f, float d, long
     return lo + (long long)(first + (h2 ? __ffs(h2) - 1 : cnt - 1));
 }
 
+// heat_bath_chain where the range has at most 32 values and the numbers are
+// small (see heat_bath_narrow): 32-bit arithmetic, the minimum by one warp
+// reduction.
+__device__ __forceinline__ int heat_bath_chain32(int f, int d, int z, int lo, uint32_t width, uint32_t xu, float beta,
+                                                 int lane) {
+    constexpr unsigned full = 0xffffffffu;
+    const int v = lo + lane;
+    const bool in = (uint32_t)lane <= width;
+    const int de = (v - z) * (f + d * (v + z));
+    const int mn = __reduce_min_sync(full, in ? de : 0);   // (0, at z, is among them)
+    const float w = expf(-(__int2float_rn(de - mn) * beta));
+    float sum = 0.f, comp = 0.f, pre = 0.f;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        if (8u * g > width) break;   // the same for every lane
+        float wi[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) wi[j] = __shfl_sync(full, w, 8 * g + j);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            // (values past the range come last and are never looked at)
+            const float y = wi[j] - comp;
+            const float t = sum + y;
+            const bool ok = (uint32_t)(8 * g + j) <= width;
+            comp = ok ? (t - sum) - y : comp;
+            sum = ok ? t : sum;
+            pre = lane == 8 * g + j ? sum : pre;
+        }
+    }
+    const float thr = unit_open_left(xu) * sum;
+    const unsigned hit = __ballot_sync(full, in && pre >= thr);
+    return lo + (hit ? __ffs(hit) - 1 : (int)width);
+}
+__device__ __forceinline__ bool small_numbers(long long f, long long d, int lo, uint32_t width) {
+    return width < 32u && f < (1 << 23) && f > -(1 << 23) && d < (1 << 10) && d > -(1 << 10) && lo > -(1 << 12) &&
+           (long long)lo + (long long)width < (1 << 12);
+}
+
 // One variable's heat-bath draw by a whole warp (out of line: four forms that
 // would each hold registers of the block loop).
 template <class F>
@@ -161,6 +201,9 @@ __device__ __noinline__ int heat_bath_in_turn(F f, F d, int z, int lo, uint32_t 
     vv.f = f;
     vv.d = d;
     if (vv.linear()) return (int)heat_bath_linear(Num<F>::to_f(f), lo, width, xu, beta);
+    if constexpr (!Num<F>::is_float)
+        if (!wide && small_numbers(f, d, lo, width))
+            return heat_bath_chain32((int)f, (int)d, z, lo, width, xu, beta, lane);
     if (wide) return (int)heat_bath_warp<F, KIND_QUIO>(vv, z, lo, width, xu, beta, lane);
     if (Num<F>::is_float && width < 256u && lo > -(1 << 22) && (long long)lo + (long long)width < (1 << 22))
         return (int)heat_bath_small_warp((float)f, (float)d, z, lo, width, xu, beta, temp, lane);
