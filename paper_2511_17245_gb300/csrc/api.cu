@@ -733,7 +733,9 @@ sa_status compile_model(sa_model* M, int32_t n, const int64_t* lower, const int6
 // variables that is waited for took about 300 us instead of 83.  The pool keeps at
 // most kPoolKeep bytes between calls and gives them back when the device's last
 // model is destroyed.  (Allocation and reuse are stream-ordered, as in the
-// default pool; where no pool can be made, the default one serves.)
+// default pool; where no pool can be made, the default one serves.  It is made
+// with the device's first model, like the model's own allocation, and not inside
+// a run, which may go on beside another thread's stream capture.)
 constexpr uint64_t kPoolKeep = 64ull << 20;
 struct DevicePool {
     cudaMemPool_t pool = nullptr;
@@ -762,8 +764,10 @@ cudaMemPool_t device_pool(int device) {
     }
     return d.pool;
 }
-// Counts the device's models; the last one to go trims the pool.
+// Counts the device's models; the first one makes the pool, the last one to go
+// trims it.
 void count_model(int device, int change) {
+    if (change > 0) device_pool(device);
     std::lock_guard<std::mutex> lk(g_pool_mu);
     DevicePool& d = g_pools[device];
     d.models += change;
