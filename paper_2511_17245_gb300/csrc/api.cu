@@ -268,7 +268,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
     struct Offs {
         size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk_w = 0, blk_i = 0;
         bool blk_wide = false;
-        size_t up_rec, adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
+        size_t up_rec, up_pair = SIZE_MAX, adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
         size_t slot_base, omega, aconst_i, aconst_f, aconst_d, inc_term, inc_exp, inc_rec, inc16 = SIZE_MAX, term_ptr, mem_var, mem_exp,
             tcoef_i, tcoef_f, tcoef_d;
     } off{};
@@ -386,6 +386,26 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
             up[4 * (size_t)i + 2] = (int32_t)(ptr[k] + deg[k]);
         }
         off.up_rec = blob.add(up);
+        int64_t n_pairs = 0;
+        for (int32_t k = 0; k < n; ++k) n_pairs += ptr[k] + deg[k] - up_first[k];
+        if (M->f32_coeffs && M->is_float && sa::plan_pair_list(n, dm.z_base, z_top, n_pairs)) {
+            std::vector<int32_t> pair;
+            bool normal = true;
+            pair.reserve(2 * (size_t)n_pairs);
+            for (int32_t k = 0; k < n; ++k)
+                for (int64_t e = up_first[k]; e < ptr[k] + deg[k]; ++e) {
+                    const float w = (float)vd[e];
+                    int32_t bits;
+                    std::memcpy(&bits, &w, 4);
+                    normal = normal && (w == 0.0f || std::isnormal(w));
+                    pair.push_back((int32_t)((uint32_t)k | ((uint32_t)col[e] << 16)));
+                    pair.push_back(bits);
+                }
+            if (normal) {
+                off.up_pair = blob.add(pair);
+                dm.n_pairs = (int32_t)n_pairs;
+            }
+        }
         if (sa::plan_block_model(n, M->n_levels)) {
             // blocked sweeps: records in index order, the earlier neighbours in
             // each variable's block of 32 and the block's couplings
@@ -616,6 +636,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         }
         dm.adj_col = at<int32_t>(b, off.adj_col);
         dm.up_rec = at<int32_t>(b, off.up_rec);
+        if (off.up_pair != SIZE_MAX) dm.up_pair = at<int32_t>(b, off.up_pair);
         if (M->is_float) {
             dm.adj_f = at<float>(b, off.adj_f);
             dm.adj_d = off.adj_d == SIZE_MAX ? nullptr : at<double>(b, off.adj_d);

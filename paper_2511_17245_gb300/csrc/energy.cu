@@ -188,20 +188,32 @@ __global__ void __launch_bounds__(256) energy_kernel(const EnergyArgs a) {
 // G states; a thread takes whole rows, four entries per vector load,
 // rows of the same length and alignment side by side (an FP64 instruction holds
 // the pipe for 16 cycles however few lanes want it).
-// What bounds it: FP64 additions (two lanes per cycle and SM), one per pair and
-// state, 0.52 ms for 4096 states of 80,000 pairs; the conversions to FP64, which
-// share that pipe, are done by moving bits.  The one-state-per-block form walked
-// every pair from both ends with a 4-byte gather from global memory each and
-// waited for the load queue (6.9 ms).
+// Sparse models with normal fp32 couplings and values within +-4095 take their
+// pairs from a flat list instead (PAIRS): a row of eight entries leaves lanes of
+// an FP64 instruction idle, and z_k z_j, a whole number below 2^24, is exact.
+// What bounds it: FP64 multiply-adds (two lanes per cycle and SM), one per pair
+// and state, 0.52 ms for 4096 states of 80,000 pairs (and 0.13 ms for the linear
+// and square terms); the conversions to FP64, which share that pipe, are done by
+// moving bits.  4096 states of 10,000 variables and 80,000 pairs, a call: one
+// state per block from both ends of every pair 6.81 ms; by rows, four states per
+// block, 1.91; from the list 1.76, and with no FP64 conversion left beside the
+// bit moves (widen_normal) 0.82.
 __device__ __forceinline__ double widen_f(float x) {
     const uint32_t u = __float_as_uint(x);
     const uint32_t e = (u >> 23) & 0xFFu;
     if (e - 1u >= 254u) return (double)x;   // zero, denormal, infinite, NaN
     return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
 }
+// The same for normal numbers and zeros alone, with no conversion beside it that
+// a compiler could issue under a false predicate.
+__device__ __forceinline__ double widen_normal(float x) {
+    const uint32_t u = __float_as_uint(x);
+    const uint32_t hi = (u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u);
+    return __hiloint2double((u << 1) == 0u ? 0 : (int)hi, (int)(u << 29));
+}
 template <class Z>
 __device__ __forceinline__ double widen_z(int z) {
-    if constexpr (sizeof(Z) < 4) return z == 0 ? 0.0 : widen_f(__int2float_rn(z));   // (below 2^24: see launch_energy)
+    if constexpr (sizeof(Z) < 4) return widen_normal(__int2float_rn(z));   // (below 2^24: see launch_energy)
     else return __int2double_rn(z);
 }
 
@@ -210,7 +222,7 @@ struct alignas(sizeof(Z) * G) ZPack {
     Z z[G];
 };
 
-template <bool IS_FLOAT, class Z, int G>
+template <bool IS_FLOAT, class Z, int G, bool PAIRS>
 __global__ void __launch_bounds__(256) quio_energy_kernel(const EnergyArgs a) {
     using Acc = typename std::conditional<IS_FLOAT, double, long long>::type;
     extern __shared__ __align__(16) uint8_t zraw[];
@@ -241,53 +253,88 @@ __global__ void __launch_bounds__(256) quio_energy_kernel(const EnergyArgs a) {
     Acc e[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) e[g] = Acc(0);
-    for (int i = threadIdx.x; i < m.n; i += blockDim.x) {
-        const int4 rec = __ldg(reinterpret_cast<const int4*>(m.up_rec) + i);
-        const int k = rec.x, first = rec.y, end = rec.z;
-        Acc f[G];
+    if constexpr (PAIRS) {
+        // z_k z_j is a whole number below 2^24: one conversion and one FP64
+        // multiply-add per pair and state, in every lane
+        constexpr int U = 4;
+        const int2* pairs = reinterpret_cast<const int2*>(m.up_pair);
+        for (int p0 = threadIdx.x; p0 < m.n_pairs; p0 += U * blockDim.x) {
+            int2 q[U];
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            if constexpr (IS_FLOAT) f[g] = m.lin_d[k];
-            else f[g] = m.lin_i[k];
-        }
-        for (int q0 = first & ~3; q0 < end; q0 += 4) {
-            const int4 c4 = __ldg(reinterpret_cast<const int4*>(m.adj_col + q0));
-            const int col[4] = {c4.x, c4.y, c4.z, c4.w};
-            Acc w[4];
-            if constexpr (IS_FLOAT) {
-                if (m.adj_d != nullptr) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) w[u] = __ldg(m.adj_d + q0 + u);
-                } else {
-                    const float4 w4 = __ldg(reinterpret_cast<const float4*>(m.adj_f + q0));
-                    w[0] = widen_f(w4.x); w[1] = widen_f(w4.y); w[2] = widen_f(w4.z); w[3] = widen_f(w4.w);
-                }
-            } else {
-                const longlong2* wp = reinterpret_cast<const longlong2*>(m.adj_i + q0);
-                const longlong2 wa = __ldg(wp), wb = __ldg(wp + 1);
-                w[0] = wa.x; w[1] = wa.y; w[2] = wb.x; w[3] = wb.y;
+            for (int u = 0; u < U; ++u) {
+                const int p = p0 + u * (int)blockDim.x;
+                q[u] = p < m.n_pairs ? __ldg(pairs + p) : make_int2(0, 0);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (q0 + u < first || q0 + u >= end) continue;
-                const ZPack<Z, G> zj = zs[col[u]];
+            for (int u = 0; u < U; ++u) {
+                if (p0 + u * (int)blockDim.x >= m.n_pairs) break;
+                const ZPack<Z, G> zk = zs[q[u].x & 0xFFFF], zj = zs[(uint32_t)q[u].x >> 16];
+                const double w = widen_normal(__int_as_float(q[u].y));
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    const int z = m.z_base + (int)(uint32_t)zj.z[g];
-                    if constexpr (IS_FLOAT) f[g] += w[u] * widen_z<Z>(z);
-                    else f[g] += w[u] * (long long)z;
+                    const int zz = (m.z_base + (int)zk.z[g]) * (m.z_base + (int)zj.z[g]);
+                    e[g] = fma(w, widen_z<Z>(zz), e[g]);
                 }
             }
         }
-        const ZPack<Z, G> zk = zs[k];
+        for (int k = threadIdx.x; k < m.n; k += blockDim.x) {
+            const double l = m.lin_d[k], d = m.diag_d[k];
+            const ZPack<Z, G> zk = zs[k];
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-            const int z = m.z_base + (int)(uint32_t)zk.z[g];
-            if constexpr (IS_FLOAT) {
-                const double zd = widen_z<Z>(z);
-                e[g] += zd * (f[g] + m.diag_d[k] * zd);
-            } else {
-                e[g] += (long long)z * (f[g] + m.diag_i[k] * (long long)z);
+            for (int g = 0; g < G; ++g) {
+                const double zd = widen_z<Z>(m.z_base + (int)zk.z[g]);
+                e[g] += zd * (l + d * zd);
+            }
+        }
+    } else {
+        for (int i = threadIdx.x; i < m.n; i += blockDim.x) {
+            const int4 rec = __ldg(reinterpret_cast<const int4*>(m.up_rec) + i);
+            const int k = rec.x, first = rec.y, end = rec.z;
+            Acc f[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                if constexpr (IS_FLOAT) f[g] = m.lin_d[k];
+                else f[g] = m.lin_i[k];
+            }
+            for (int q0 = first & ~3; q0 < end; q0 += 4) {
+                const int4 c4 = __ldg(reinterpret_cast<const int4*>(m.adj_col + q0));
+                const int col[4] = {c4.x, c4.y, c4.z, c4.w};
+                Acc w[4];
+                if constexpr (IS_FLOAT) {
+                    if (m.adj_d != nullptr) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) w[u] = __ldg(m.adj_d + q0 + u);
+                    } else {
+                        const float4 w4 = __ldg(reinterpret_cast<const float4*>(m.adj_f + q0));
+                        w[0] = widen_f(w4.x); w[1] = widen_f(w4.y); w[2] = widen_f(w4.z); w[3] = widen_f(w4.w);
+                    }
+                } else {
+                    const longlong2* wp = reinterpret_cast<const longlong2*>(m.adj_i + q0);
+                    const longlong2 wa = __ldg(wp), wb = __ldg(wp + 1);
+                    w[0] = wa.x; w[1] = wa.y; w[2] = wb.x; w[3] = wb.y;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (q0 + u < first || q0 + u >= end) continue;
+                    const ZPack<Z, G> zj = zs[col[u]];
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const int z = m.z_base + (int)(uint32_t)zj.z[g];
+                        if constexpr (IS_FLOAT) f[g] += w[u] * widen_z<Z>(z);
+                        else f[g] += w[u] * (long long)z;
+                    }
+                }
+            }
+            const ZPack<Z, G> zk = zs[k];
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                const int z = m.z_base + (int)(uint32_t)zk.z[g];
+                if constexpr (IS_FLOAT) {
+                    const double zd = widen_z<Z>(z);
+                    e[g] += zd * (f[g] + m.diag_d[k] * zd);
+                } else {
+                    e[g] += (long long)z * (f[g] + m.diag_i[k] * (long long)z);
+                }
             }
         }
     }
@@ -302,9 +349,9 @@ __global__ void __launch_bounds__(256) quio_energy_kernel(const EnergyArgs a) {
     }
 }
 
-template <bool IS_FLOAT, class Z, int G>
+template <bool IS_FLOAT, class Z, int G, bool PAIRS>
 int launch_quio_energy(const EnergyArgs& a, cudaStream_t st) {
-    auto kern = quio_energy_kernel<IS_FLOAT, Z, G>;
+    auto kern = quio_energy_kernel<IS_FLOAT, Z, G, PAIRS>;
     const size_t sh = (size_t)a.m.n * sizeof(Z) * G;
     if (sh > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
@@ -314,13 +361,20 @@ int launch_quio_energy(const EnergyArgs& a, cudaStream_t st) {
     return (int)cudaGetLastError();
 }
 
+template <bool IS_FLOAT, class Z, int G>
+int launch_quio_form(const EnergyArgs& a, cudaStream_t st) {
+    if constexpr (IS_FLOAT && sizeof(Z) < 4)
+        if (a.m.up_pair != nullptr) return launch_quio_energy<IS_FLOAT, Z, G, true>(a, st);
+    return launch_quio_energy<IS_FLOAT, Z, G, false>(a, st);
+}
+
 // Four states per block when that still gives every SM a few blocks and they
 // fit, else one; returns false when one state does not fit on chip.
 template <bool IS_FLOAT, class Z>
 bool quio_energy_shape(const EnergyArgs& a, cudaStream_t st, int& rc) {
     const size_t room = (size_t)sweep_max_shared_optin() - 1024, one = (size_t)a.m.n * sizeof(Z);
-    if (4 * one <= room && a.n_states >= 4 * 304) rc = launch_quio_energy<IS_FLOAT, Z, 4>(a, st);
-    else if (one <= room) rc = launch_quio_energy<IS_FLOAT, Z, 1>(a, st);
+    if (4 * one <= room && a.n_states >= 4 * 304) rc = launch_quio_form<IS_FLOAT, Z, 4>(a, st);
+    else if (one <= room) rc = launch_quio_form<IS_FLOAT, Z, 1>(a, st);
     else return false;
     return true;
 }

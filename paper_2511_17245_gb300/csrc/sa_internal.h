@@ -59,6 +59,10 @@ struct DevModel {
     // the number of those entries (descending) and the first one's place in its
     // group of four, so that a warp's lanes walk alike
     const int32_t* up_rec;
+    // normal fp32 couplings of sparse models with small values (plan_pair_list): every
+    // pair once, {smaller variable | larger << 16, fp32 bits of J}, by rows; null otherwise
+    const int32_t* up_pair;
+    int32_t n_pairs;
     int32_t z_base;             // smallest lower bound
     uint32_t z_span;            // largest upper bound minus z_base
     const int32_t* adj_col;     // symmetric adjacency, both directions
@@ -290,6 +294,14 @@ inline bool plan_block_model(int32_t n, int32_t n_levels) { return (int64_t)n <=
 inline bool plan_blocked(const PlanModel& m, int rule, bool allowed) {
     if (!m.block_model || !allowed) return false;
     return rule != RULE_HEAT_BATH || (int64_t)m.n <= (int64_t)kBlockWidthHeat * m.n_levels;
+}
+
+// Whether the model holds the pair list that the energies of states are summed
+// from: variables in 16 bits, values whose product two of them have exactly in
+// fp32, and short rows (rows of 64 entries and more fill a thread's groups of
+// four without it, and the list of a complete graph would be half its adjacency).
+inline bool plan_pair_list(int32_t n, int64_t lo, int64_t hi, int64_t pairs) {
+    return n <= 65536 && lo > -4096 && hi < 4096 && pairs <= 32 * (int64_t)n;
 }
 
 // Bytes of one block staged on chip: couplings (32 x 32 x 4), records, masks.

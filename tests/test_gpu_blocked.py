@@ -104,6 +104,25 @@ def test_carries_between_the_words_of_a_field(scale):
         assert torch.equal(out["energies"], model.energy(out["states"]))
 
 
+@pytest.mark.parametrize("n,edges", [(2, 1), (40, 255), (40, 257), (300, 1025), (70, 2240), (70, 2241), (65536, 70000),
+                                     (65537, 70000)])
+@pytest.mark.parametrize("lo,hi", [(-1, 1), (0, 255), (-4095, 4095), (-4096, 4095)])
+def test_energies_from_the_pair_list(n, edges, lo, hi):
+    """Around the limits of the pair list (variables, values, row lengths), of a
+    thread's four pairs and of the states per block."""
+    inst = wl.quio_sparse_wide(5, n=n, n_edges=edges, lo=lo, hi=hi)
+    model = Model(inst)
+    c = inst["coeffs"].astype(np.float64)
+    pairs = inst["term_vars"][3 * n:].reshape(-1, 2)
+    for n_states in ((3,) if n > 1000 else (3, 1217)):
+        states = wl.initial_states(4, inst, n_states)
+        got = model.energy(torch.from_numpy(states).cuda()).cpu().numpy()
+        z = states.astype(np.float64)
+        terms = np.concatenate([z * c[:n], z * z * c[n:2 * n], z[:, pairs[:, 0]] * z[:, pairs[:, 1]] * c[2 * n:]], axis=1)
+        bound = (terms.shape[1] + 4) * 2.0 ** -52 * np.abs(terms).sum(axis=1)
+        assert np.all(np.abs(got - terms.sum(axis=1)) <= bound)
+
+
 @pytest.mark.parametrize("n_states", [1, 5, 1215, 1216, 1219])
 @pytest.mark.parametrize("lo,hi,coef", [(0, 255, "f32"), (-300, 300, "i32"), (-40, 90000, "f64"),
                                         (-(1 << 25), 1 << 25, "f64")])
