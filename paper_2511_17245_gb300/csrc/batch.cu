@@ -66,7 +66,7 @@ struct sa_batch {
     uint8_t* d_gstate = nullptr;
     size_t gstate_bytes = 0;
     int rpc = 0, tpr = 0, blocks = 0;
-    size_t slot_bytes = 0;
+    size_t slot_bytes = 0, shared_bytes = 0;
     bool smem = true;
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -93,29 +93,18 @@ sa_status apply_shape(sa_batch* b, int tpr, int rpc_req) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
     size_t slot = 0;
     for (int i = 0; i < b->n; ++i) slot = std::max(slot, layout(b->h_insts[i], b->views[i], b->zbytes, tpr));
-    const int smem_max = sa::sweep_max_shared_optin() - 8192;   // leave room for the static argument copies
-    int fit = (int)((size_t)std::max(0, smem_max) / slot);
-    fit = std::min(fit, std::min(15, 512 / tpr));
-    bool smem = fit >= 1;
-    int rpc = rpc_req > 0 ? rpc_req : (smem ? fit : std::min(15, 512 / tpr));
-    if (rpc < 1 || rpc > 15 || rpc * tpr > 512) return bfail(SA_ERR_INVALID, "batch launch shape out of range");
-    if (smem && rpc > fit) return bfail(SA_ERR_INVALID, "replicas_per_block exceeds shared memory");
-    // persistent grid: as many blocks as fit on the GPU at once (1 per SM with large shared use)
-    int per_sm = 1;
-    if (smem) per_sm = std::max(1, std::min((int)((size_t)sa::sweep_max_shared_optin() / ((size_t)rpc * slot + 8192)),
-                                            2048 / (rpc * tpr)));
-    else per_sm = std::max(1, 2048 / (rpc * tpr));
-    per_sm = std::min(per_sm, std::max(1, 65536 / (rpc * tpr * 128)));   // registers: up to 128 per thread
-    // blocked instances stage their blocks behind the regions where there is room
     bool any_blocked = false;
     for (const auto& a : b->h_insts) any_blocked = any_blocked || a.blocked;
-    if (smem && any_blocked && (size_t)rpc * (slot + 2 * sa::kBlockStage) <= (size_t)std::max(0, smem_max) &&
-        std::max(1, (int)((size_t)sa::sweep_max_shared_optin() / ((size_t)rpc * (slot + 2 * sa::kBlockStage) + 8192))) >= per_sm) {
+    sa::BatchShape sh{};
+    if (const char* err = sa::plan_batch_shape((int64_t)slot, tpr, rpc_req, any_blocked, sa::sweep_max_shared_optin(), &sh))
+        return bfail(SA_ERR_INVALID, err);
+    if (sh.staged)
         for (auto& a : b->h_insts)
             if (a.blocked) a.off_blk = (int32_t)slot;
-        slot += 2 * sa::kBlockStage;
-    }
-    int blocks = sms * per_sm;
+    slot = (size_t)sh.slot_bytes;
+    const int rpc = sh.rpc;
+    const bool smem = sh.in_global == 0;
+    int blocks = sms * sh.per_sm;
     const int need = (int)((b->h_units.size() + rpc - 1) / rpc);
     blocks = std::max(1, std::min(blocks, need));
     if (!smem) {
@@ -133,6 +122,7 @@ sa_status apply_shape(sa_batch* b, int tpr, int rpc_req) {
     b->rpc = rpc;
     b->blocks = blocks;
     b->slot_bytes = slot;
+    b->shared_bytes = (size_t)sh.shared_bytes;
     b->smem = smem;
     for (auto& a : b->h_insts) a.rpc = rpc;
     cudaError_t e = cudaMemcpy(b->d_insts, b->h_insts.data(), sizeof(sa::SweepArgs) * b->n, cudaMemcpyHostToDevice);
@@ -153,8 +143,6 @@ sa::BatchArgs batch_args(const sa_batch* b, const sa::SweepArgs* insts) {
     return a;
 }
 
-size_t shared_bytes(const sa_batch* b) { return b->smem ? (size_t)b->rpc * b->slot_bytes : 0; }
-
 sa_status capture(sa_batch* b) {
     if (b->exec) {
         cudaGraphExecDestroy(b->exec);
@@ -162,14 +150,14 @@ sa_status capture(sa_batch* b) {
     }
     const sa::BatchArgs a = batch_args(b, b->d_insts);
     int le = sa::launch_batch(a, b->is_float, b->kind, b->zbytes, b->rule, b->smem, 0, b->rpc * b->tpr,
-                              shared_bytes(b), b->cap, true);
+                              b->shared_bytes, b->cap, true);
     if (le != 0) return bcuda((cudaError_t)le, "batch kernel attributes");
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return bcuda(e, "begin capture");
     cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned int), b->cap);
     le = sa::launch_batch(a, b->is_float, b->kind, b->zbytes, b->rule, b->smem, b->blocks, b->rpc * b->tpr,
-                          shared_bytes(b), b->cap, false);
+                          b->shared_bytes, b->cap, false);
     e = cudaStreamEndCapture(b->cap, &g);
     if (le != 0) return bcuda((cudaError_t)le, "batch kernel capture");
     if (e != cudaSuccess) return bcuda(e, "end capture");
@@ -376,7 +364,7 @@ sa_status sa_batch_autotune(sa_batch* b, int32_t trial_sweeps, void* stream) {
             cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned int), st);
             cudaEventRecord(e0, st);
             int le = sa::launch_batch(a, b->is_float, b->kind, b->zbytes, b->rule, b->smem, b->blocks,
-                                      b->rpc * b->tpr, shared_bytes(b), st, true);
+                                      b->rpc * b->tpr, b->shared_bytes, st, true);
             cudaEventRecord(e1, st);
             if (le != 0) break;
             cudaEventSynchronize(e1);

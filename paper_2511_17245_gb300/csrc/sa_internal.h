@@ -450,6 +450,54 @@ inline const char* plan_run(const PlanModel& m, int rule, bool allow_blocks, int
     return nullptr;
 }
 
+// ------------------------------------------------------------------ batch launch shape
+// One thread group's place in a batch kernel besides its replica's state: the
+// arguments of its present instance and the unit it claimed.  They lie in the
+// dynamic shared memory behind the state regions, one per group of the launch, so
+// that what the shape counts is what the kernel uses.
+struct alignas(16) BatchGroup {
+    SweepArgs args;
+    int32_t unit;
+};
+
+struct BatchShape {
+    int32_t rpc, per_sm;        // replicas per block, blocks per SM of the persistent grid
+    int32_t in_global;          // replica state in global slabs
+    int32_t staged;             // blocked instances stage their blocks behind the region
+    int64_t slot_bytes;         // bytes of one replica's region
+    int64_t shared_bytes;       // dynamic shared memory of one block
+};
+
+// Shape of a batch launch whose largest replica region takes `slot` bytes at
+// `tpr` threads per replica.  rpc_req <= 0: as many replicas per block as shared
+// memory and 512 threads allow.
+inline const char* plan_batch_shape(int64_t slot, int tpr, int rpc_req, bool any_blocked, int64_t smem_max,
+                                    BatchShape* p) {
+    constexpr int64_t group = (int64_t)sizeof(BatchGroup);
+    const int cap = 15 < 512 / tpr ? 15 : 512 / tpr;
+    const int64_t room = smem_max / (slot + group);
+    const int fit = room < cap ? (int)room : cap;
+    p->in_global = fit < 1 ? 1 : 0;
+    p->rpc = rpc_req > 0 ? rpc_req : (p->in_global ? cap : fit);
+    if (p->rpc < 1 || p->rpc > 15 || p->rpc * tpr > 512) return "batch launch shape out of range";
+    if (!p->in_global && p->rpc > fit) return "replicas_per_block exceeds shared memory";
+    // persistent grid: as many blocks as fit on the GPU at once (1 per SM with
+    // large shared use; 1 KB of each block is the system's), registers for up to
+    // 128 per thread
+    auto shared = [&](int64_t s) { return (p->in_global ? 0 : p->rpc * s) + p->rpc * group; };
+    auto fits = [&](int64_t s) { return (int)((smem_max + 1024) / (shared(s) + 1024)); };
+    int per_sm = 2048 / (p->rpc * tpr);
+    if (per_sm > 65536 / (p->rpc * tpr * 128)) per_sm = 65536 / (p->rpc * tpr * 128);
+    if (per_sm > fits(slot)) per_sm = fits(slot);
+    p->per_sm = per_sm < 1 ? 1 : per_sm;
+    // blocked instances stage their blocks where there is room
+    p->staged = any_blocked && !p->in_global && shared(slot + 2 * kBlockStage) <= smem_max &&
+                fits(slot + 2 * kBlockStage) >= p->per_sm;
+    p->slot_bytes = slot + (p->staged ? 2 * kBlockStage : 0);
+    p->shared_bytes = shared(p->slot_bytes);
+    return nullptr;
+}
+
 // ------------------------------------------------------------------ time-sliced runs
 // When R replicas exceed the P thread groups that can be resident at once, a
 // plain launch runs ceil(R / P) waves and the last one leaves slots idle.  A

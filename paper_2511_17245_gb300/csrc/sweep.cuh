@@ -2036,34 +2036,32 @@ __device__ __noinline__ void batch_body(const SweepArgs& a, int slot, int t, int
 template <class F, class Z, int RULE, int KIND, bool SMEM>
 __global__ void __launch_bounds__(512, 1) batch_kernel(const BatchArgs b) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    __shared__ SweepArgs args_s[15];
-    __shared__ int unit_s[15];
     const int slot = threadIdx.x / b.tpr;
     const int t = threadIdx.x - slot * b.tpr;
     if (slot >= b.rpc) return;
     const int bar_id = 1 + slot;
+    BatchGroup& g = reinterpret_cast<BatchGroup*>(smem_raw + (SMEM ? (size_t)b.rpc * (size_t)b.slot_bytes : 0))[slot];
     uint8_t* base = SMEM ? (smem_raw + (size_t)slot * (size_t)b.slot_bytes)
                          : (b.gstate + ((size_t)blockIdx.x * b.rpc + slot) * (size_t)b.slot_bytes);
     for (;;) {
-        if (t == 0) unit_s[slot] = (int)atomicAdd(b.counter, 1u);
+        if (t == 0) g.unit = (int)atomicAdd(b.counter, 1u);
         named_bar(bar_id, b.tpr);
-        const int u = unit_s[slot];
+        const int u = g.unit;
         if (u >= b.n_units) break;
         const BatchUnit un = b.units[u];
         const uint32_t* src = reinterpret_cast<const uint32_t*>(b.insts + un.inst);
-        uint32_t* dst = reinterpret_cast<uint32_t*>(&args_s[slot]);
+        uint32_t* dst = reinterpret_cast<uint32_t*>(&g.args);
         for (int w = t; w < (int)(sizeof(SweepArgs) / 4); w += b.tpr) dst[w] = src[w];
         named_bar(bar_id, b.tpr);
         if constexpr (KIND == KIND_QUIO) {
-            if (args_s[slot].blocked)
-                batch_body<F, Z, RULE, KIND, SMEM, true>(args_s[slot], slot, t, un.replica, b.slot_bytes, base);
+            if (g.args.blocked)
+                batch_body<F, Z, RULE, KIND, SMEM, true>(g.args, slot, t, un.replica, b.slot_bytes, base);
             else
-                batch_body<F, Z, RULE, KIND, SMEM, false>(args_s[slot], slot, t, un.replica, b.slot_bytes, base);
+                batch_body<F, Z, RULE, KIND, SMEM, false>(g.args, slot, t, un.replica, b.slot_bytes, base);
         } else {
-            replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL, false>(args_s[slot], slot, t, un.replica,
-                                                                                   base);
+            replica_body<F, Z, RULE, KIND, SMEM ? MEM_SHARED : MEM_GLOBAL, false>(g.args, slot, t, un.replica, base);
         }
-        named_bar(bar_id, b.tpr);   // the group is done with args_s and unit_s
+        named_bar(bar_id, b.tpr);   // the group is done with its arguments and unit
     }
 }
 

@@ -168,3 +168,35 @@ def test_plan_run_threads(tmp_path, n, levels, dense, links, R, rule, want):
     assert tuple(out[:3]) == want
     assert out[3] == want[0] and out[4] == 0     # the level order runs with the same threads
     assert out[5:] == [64, 64]
+
+
+def test_batch_shapes_count_the_argument_copies(tmp_path):
+    """Every batch shape, over region sizes up to past a block's shared memory,
+    all thread counts and both forms: the dynamic shared memory (the kernel has no
+    other) holds the regions and one argument record per group within the limit,
+    staging never lowers the blocks per SM, and a region that fits with its record
+    stays on chip."""
+    body = """
+  const int64_t optin = 232448, group = sizeof(sa::BatchGroup);
+  int bad = 0, seen = 0;
+  for (int tpr = 32; tpr <= 512; tpr += 32)
+    for (int64_t slot = 2048; slot <= optin + 1024; slot += 16)
+      for (int blk = 0; blk < 2; ++blk) {
+        sa::BatchShape s{};
+        if (sa::plan_batch_shape(slot, tpr, 0, blk != 0, optin, &s)) { ++bad; continue; }
+        ++seen;
+        const int64_t want = (s.in_global ? 0 : s.rpc * s.slot_bytes) + s.rpc * group;
+        bad += s.shared_bytes != want || s.shared_bytes > optin || s.rpc * tpr > 512 || s.per_sm < 1;
+        bad += (s.in_global != 0) != (slot + group > optin);
+        bad += s.slot_bytes != slot + (s.staged ? 2 * sa::kBlockStage : 0) || (s.staged && (!blk || s.in_global));
+        sa::BatchShape plain{};
+        sa::plan_batch_shape(slot, tpr, 0, false, optin, &plain);
+        bad += plain.rpc != s.rpc || plain.per_sm != s.per_sm;
+        sa::BatchShape over{};
+        if (!s.in_global && s.rpc < 15 && (s.rpc + 1) * tpr <= 512)
+          bad += sa::plan_batch_shape(slot, tpr, s.rpc + 1, false, optin, &over) == nullptr;
+      }
+  std::printf("%d %d %d\\n", bad, seen, (int)(group % 16));
+"""
+    bad, seen, rem = (int(x) for x in _compile_and_run(tmp_path, body))
+    assert bad == 0 and rem == 0 and seen > 400_000
