@@ -349,14 +349,18 @@ __global__ void __launch_bounds__(256) quio_energy_kernel(const EnergyArgs a) {
     }
 }
 
+// Dynamic shared memory that a block may have beside its reduction scratch.
+size_t energy_room() { return (size_t)sweep_max_shared_optin() - 1024; }
+
 template <bool IS_FLOAT, class Z, int G, bool PAIRS>
 int launch_quio_energy(const EnergyArgs& a, cudaStream_t st) {
     auto kern = quio_energy_kernel<IS_FLOAT, Z, G, PAIRS>;
     const size_t sh = (size_t)a.m.n * sizeof(Z) * G;
-    if (sh > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-        if (e != cudaSuccess) return (int)e;
-    }
+    // one limit for every call and size: what a launch may use without it counts
+    // static and dynamic bytes, and a limit of this call's size could be lowered by
+    // another thread's call between here and the launch
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)energy_room());
+    if (e != cudaSuccess) return (int)e;
     kern<<<(unsigned)((a.n_states + G - 1) / G), 256, sh, st>>>(a);
     return (int)cudaGetLastError();
 }
@@ -372,7 +376,7 @@ int launch_quio_form(const EnergyArgs& a, cudaStream_t st) {
 // fit, else one; returns false when one state does not fit on chip.
 template <bool IS_FLOAT, class Z>
 bool quio_energy_shape(const EnergyArgs& a, cudaStream_t st, int& rc) {
-    const size_t room = (size_t)sweep_max_shared_optin() - 1024, one = (size_t)a.m.n * sizeof(Z);
+    const size_t room = energy_room(), one = (size_t)a.m.n * sizeof(Z);
     if (4 * one <= room && a.n_states >= 4 * 304) rc = launch_quio_form<IS_FLOAT, Z, 4>(a, st);
     else if (one <= room) rc = launch_quio_form<IS_FLOAT, Z, 1>(a, st);
     else return false;

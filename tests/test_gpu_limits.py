@@ -52,3 +52,29 @@ def test_batch_shapes_that_fill_shared_memory(n):
     ref = model.run("metropolis", 6, 40, seed=9)
     assert np.array_equal(st, ref["states"].cpu().numpy())
     assert np.array_equal(en, ref["energies"].cpu().numpy())
+
+
+@pytest.mark.parametrize("n,hi,n_states", [(12288, 255, 1216), (12273, 255, 1216), (6144, 300, 1216), (6137, 300, 1216),
+                                           (49152, 255, 3), (49089, 255, 3), (24576, 300, 3), (12288, 255, 3)])
+def test_energies_at_48_kb_of_staged_states(n, hi, n_states):
+    """Staged states of 48 KB and the first size whose static scratch reaches past
+    it, in a process that has made no larger call: whole numbers, exact."""
+    code = f"""
+import sys; sys.path.insert(0, {ROOT!r})
+import numpy as np, torch
+from paper_2511_17245_gb300 import Model
+rng = np.random.default_rng(1)
+n, hi = {n}, {hi}
+i = np.arange(n - 1)
+inst = dict(n_vars=n, lower=np.zeros(n, np.int64), upper=np.full(n, hi, np.int64), coef_type="i32",
+            term_offsets=np.concatenate([np.arange(n + 1), n + 2 * np.arange(1, n)]).astype(np.int64),
+            term_vars=np.concatenate([np.arange(n), np.stack([i, i + 1], 1).ravel()]).astype(np.int32),
+            coeffs=rng.integers(-9, 10, 2 * n - 1).astype(np.int32))
+z = rng.integers(0, hi + 1, ({n_states}, n))
+c = inst["coeffs"].astype(np.int64)
+want = z @ c[:n] + (z[:, :-1] * z[:, 1:]) @ c[n:]
+got = Model(inst).energy(torch.from_numpy(z.astype(np.int32)).cuda()).cpu().numpy()
+assert np.array_equal(got, want), (got, want)
+"""
+    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
