@@ -79,8 +79,17 @@ __device__ __forceinline__ long long heat_bath_chain(const VarView<F, KIND_QUIO>
             const uint32_t i0 = c0 + (uint32_t)(32 * h + lane);
             float w = 0.f;
             if (i0 <= c1) {
-                if constexpr (Num<F>::is_float) w = ex2_ftz(fmaf(-vv.delta_ff(zf, v0f + (float)i0), b2, mb));
-                else w = expf(-(Num<F>::to_f(vv.delta(z, lo + (long long)i0) - mn) * beta));
+                if constexpr (Num<F>::is_float) {
+                    // the value that the scalar form reaches by steps of 1 from
+                    // its block of 32; beyond 2^24 the steps round
+                    const float first = v0f + (float)(c0 + 32u * h);
+                    float vf = first + (float)lane;
+                    if (!(fabsf(first) < 16777216.f - 32.f)) {
+                        vf = first;
+                        for (int i = 0; i < lane; ++i) vf += 1.f;
+                    }
+                    w = ex2_ftz(fmaf(-vv.delta_ff(zf, vf), b2, mb));
+                } else w = expf(-(Num<F>::to_f(vv.delta(z, lo + (long long)i0) - mn) * beta));
             }
             const int cnt = min(32, n - 32 * h);
 #pragma unroll 4
