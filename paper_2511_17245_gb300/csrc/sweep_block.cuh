@@ -476,6 +476,15 @@ __device__ __forceinline__ BlockLane<F> block_lane(const SweepArgs& a, const Z* 
     return q;
 }
 
+// Energy changes of a sweep: where every level holds one variable one lane sums
+// them in the visiting order, which is the level order's sum; elsewhere every lane
+// sums its own variables' changes, as the threads of a level do (one fp32 sum of
+// a sweep's changes had four to nine times the rounding error for levels of 5 to 16).
+template <class F>
+__device__ __forceinline__ bool sum_in_order(const DevModel& m) {
+    return Num<F>::is_float && m.n_levels == m.n;
+}
+
 // Decides block b (warp-collective) from the lanes' fields; on return f holds
 // every change of the block, the list its commits.  Returns their number.
 template <class F, class Z, int RULE>
@@ -522,7 +531,7 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
                                                 (wide >> p) & 1u);
             if (vp != zp) {
                 const int dz = vp - zp;
-                if (lane == 0) {
+                if (lane == (sum_in_order<F>(m) ? 0 : p)) {
                     const F dp = vv.delta(zp, vp);
                     if constexpr (Num<F>::is_float) acc.de = __fadd_rn(acc.de, (float)dp);   // (no fused multiply-add)
                     else acc.e += dp;
@@ -612,9 +621,10 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
             zs[q.k] = (Z)(v - (long long)q.lo);
             ++acc.changes;
             if constexpr (!Num<F>::is_float) acc.e += de;
+            else if (!sum_in_order<F>(m)) acc.de = __fadd_rn(acc.de, (float)de);
         }
-        if constexpr (Num<F>::is_float) {   // summed in the visiting order, by one lane, four at a time
-            for (unsigned c = changed; c;) {
+        if constexpr (Num<F>::is_float) {   // else by one lane, four at a time
+            for (unsigned c = sum_in_order<F>(m) ? changed : 0u; c;) {
                 float ep[4];
                 bool on[4];
 #pragma unroll
