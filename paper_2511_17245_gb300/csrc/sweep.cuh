@@ -497,9 +497,10 @@ __device__ __forceinline__ void hb_quio_window(const VarView<F, KIND_QUIO>& vv, 
         vstar = (long long)qv;
     } else {
         vstar = floor_div(-vv.f, 2 * vv.d);
-        if (vstar < lo) vstar = lo;
-        if (vstar > lo + (long long)width) vstar = lo + (long long)width;
     }
+    // (in integers: beyond 2^24 the float of a bound can lie outside of the range)
+    if (vstar < lo) vstar = lo;
+    if (vstar > lo + (long long)width) vstar = lo + (long long)width;
     const uint32_t bm = (uint32_t)(vstar - lo) / B;
     if (!kept(bm)) return;  // rounding: keep every block
     uint32_t a = 0, c = bm;  // first kept block in [0, bm]
