@@ -306,8 +306,8 @@ __device__ __noinline__ void add_commits(const DevModel& m, F* cache_any, const 
     }
 }
 
-// The commits' rows by columns, any graph: every thread of `nt` takes the next
-// (commit, link) pair.  Columns of block `own` already have the change.
+// The commits' rows by columns, integer fields of any graph: every thread of `nt`
+// takes the next (commit, link) pair.  Columns of block `own` already have the change.
 template <class F, int MEM>
 __device__ __noinline__ void scatter_commits(const DevModel& m, F* cache_any, const Commit* list_any, int count, int own,
                                              int t, int nt) {
@@ -346,35 +346,101 @@ __device__ __noinline__ void scatter_commits(const DevModel& m, F* cache_any, co
             }
 #pragma unroll
         for (int u = 0; u < 2; ++u)
-            if (at[u] >= 0 && (col[u] >> 5) != own) {
-                if constexpr (Num<F>::is_float) atomic_add_field<MEM>(cache + col[u], wt[u] * (float)dz[u]);
-                else atomic_add_field<MEM>(cache + col[u], wt[u] * (long long)dz[u]);
-            }
+            if (at[u] >= 0 && (col[u] >> 5) != own) atomic_add_field<MEM>(cache + col[u], wt[u] * (F)dz[u]);
     }
 }
 
-// Rows with fewer links than this in all are scattered by the deciding warp.
-constexpr int kScatterAlone = 96;
-
-// The commits' rows by the `nt` threads t = 0..nt-1.  `ordered`: one commit
-// after the other (bar_id < 0: the threads are one warp).
-template <class F, int MEM>
-__device__ __forceinline__ void group_scatter(const DevModel& m, F* cache, const Commit* list, int count, int own,
-                                              bool ordered, int bar_id, int t, int nt) {
-    if (!ordered) {
-        scatter_commits<F, MEM>(m, cache, list, count, own, t, nt);
-        return;
+// fp32 fields of any graph: every field takes its changes in the order of the
+// commits, so that a run's results do not depend on its threads.  Each of `nw`
+// warps owns a range of columns and walks the commits over its part of their rows
+// (rows are sorted by column), 32 links at a time with plain reads and writes;
+// eight such pieces are loaded before the first is added.
+// What bounds it: a shared-memory round trip per piece and an L2 one per eight.
+template <int MEM>
+__device__ __noinline__ void ordered_commits(const DevModel& m, float* cache_any, const Commit* list_any, int count,
+                                             int own, int warp, int nw, int lane) {
+    constexpr unsigned full = 0xffffffffu;
+    constexpr int U = 8;
+    float* cache = in_shared<MEM>(cache_any);
+    const Commit* list = in_shared<MEM>(list_any);
+    // lane c: commit c's part of this warp's columns, [row + first, row + last)
+    const Commit e = list[lane];   // (entries beyond the count are read and not used)
+    const int row = e.z;
+    int first = 0, last = lane < count ? e.w : 0;
+    if (nw > 1) {
+        const int per = (((m.n + 31) >> 5) + nw - 1) / nw * 32;
+        // the row's first entry whose column is c or above; columns are distinct,
+        // which leaves few candidates in a nearly full row
+        auto find = [&](int c) -> int {
+            int a = max(0, last - max(0, m.n - c)), b = min(last, c);
+            while (a < b) {
+                const int mid = (a + b) >> 1;
+                if (__ldg(m.adj_col + row + mid) < c) a = mid + 1;
+                else b = mid;
+            }
+            return a;
+        };
+        first = find(warp * per);
+        last = find((warp + 1) * per);
     }
-    for (int c = 0; c < count; ++c) {
-        const Commit e = list[c];
-        for (int i = t; i < e.w; i += nt) {
-            const int col = __ldg(m.adj_col + e.z + i);
-            if ((col >> 5) != own) solo_add(cache + col, Coef<F>::adj(m, e.z + i), e.y);
+    const int pieces = (last - first + 31) >> 5;
+    int upto = pieces;   // pieces of commits 0..lane
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(full, upto, o);
+        if (lane >= o) upto += u;
+    }
+    const int total = __shfl_sync(full, upto, 31);
+    for (int i0 = 0; i0 < total; i0 += U) {
+        int col[U], dz[U];
+        float w[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            col[u] = -1;
+            dz[u] = 0;
+            w[u] = 0.f;
+            if (i0 + u < total) {
+                const int h = __popc(__ballot_sync(full, upto <= i0 + u));   // the piece's commit
+                const int at = __shfl_sync(full, first - 32 * (upto - pieces), h) + 32 * (i0 + u) + lane;
+                const int end = __shfl_sync(full, last, h);
+                const int base = __shfl_sync(full, row, h);
+                dz[u] = __shfl_sync(full, e.y, h);
+                if (at < end) {
+                    col[u] = __ldg(m.adj_col + base + at);
+                    w[u] = Coef<float>::adj(m, base + at);
+                }
+            }
         }
-        if (c + 1 < count) {
-            if (bar_id < 0) __syncwarp();
-            else named_bar(bar_id, nt);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i0 + u >= total) break;
+            if (col[u] >= 0 && (col[u] >> 5) != own) solo_add(cache + col[u], w[u], dz[u]);
+            __syncwarp();   // a column may come again in the next commit
         }
+    }
+}
+
+// Integer rows with fewer links than this in all are scattered by the deciding
+// warp, and fp32 rows with fewer pieces than this beyond one per commit.
+constexpr int kScatterAlone = 96;
+constexpr int kPiecesAlone = 16;
+
+// The commits' rows by the `nt` threads t = 0..nt-1.
+template <class F, int MEM>
+__device__ __forceinline__ void group_scatter(const DevModel& m, F* cache, const Commit* list, int count, int own, int t,
+                                              int nt) {
+    if constexpr (Num<F>::is_float) {
+        // as many warps as the longest row has pieces
+        int nw = nt >> 5;
+        if (nw > 1) {
+            const int lane = t & 31;
+            const int longest = __reduce_max_sync(0xffffffffu, lane < count ? list[lane].w : 0);
+            nw = min(nw, (longest + 31) >> 5);
+            if ((t >> 5) >= nw) return;
+        }
+        ordered_commits<MEM>(m, cache, list, count, own, t >> 5, nw, t & 31);
+    } else {
+        scatter_commits<F, MEM>(m, cache, list, count, own, t, nt);
     }
 }
 
@@ -668,8 +734,7 @@ __device__ __forceinline__ void prepare_block(const SweepArgs& a, const Z* zs, u
 // on them.  One barrier per block.
 // Other graphs: warp 0 decides, then the group scatters the block's rows by
 // their columns; short rows are scattered by warp 0 without waking the others.
-// Float models whose every level holds one variable keep the order of the
-// additions (one commit at a time).
+// fp32 fields take their changes in the visiting order (see ordered_commits).
 template <class F, class Z, int RULE, int MEM>
 __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache, int* ctl, Commit* lists, uint8_t* stage,
                                             int bar_id, int t, int tpr, int r, int s, bool flush, SweepAcc<F>& acc,
@@ -751,7 +816,6 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
     } else {
         // commands to the other warps: {commits or -1, their block}, in two
         // alternating places, so that one is read before it is written again
-        const bool ordered = Num<F>::is_float && m.n_levels == m.n;
         if (t < 32) {
             for (int b = 0; b < nb; ++b) {
                 const int k = b * 32 + lane;
@@ -761,18 +825,25 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
                 if (k < m.n) cache[k] = f;
                 __syncwarp();
                 if (cnt == 0 || nb == 1) continue;
-                const int links = __reduce_add_sync(0xffffffffu, lane < cnt ? lists[lane].w : 0);
-                if (tpr > 32 && links > kScatterAlone) {
+                bool together = false;
+                if (tpr > 32) {
+                    const int len = lane < cnt ? lists[lane].w : 0;
+                    if constexpr (Num<F>::is_float)
+                        together = __reduce_add_sync(0xffffffffu, (len + 31) >> 5) - cnt > kPiecesAlone;
+                    else
+                        together = __reduce_add_sync(0xffffffffu, len) > kScatterAlone;
+                }
+                if (together) {
                     if (lane == 0) {
                         ctl[4 + 2 * acc.par] = cnt;
                         ctl[5 + 2 * acc.par] = b;
                     }
                     acc.par ^= 1;
                     named_bar(bar_id, tpr);
-                    group_scatter<F, MEM>(m, cache, lists, cnt, b, ordered, bar_id, t, tpr);
+                    group_scatter<F, MEM>(m, cache, lists, cnt, b, t, tpr);
                     named_bar(bar_id, tpr);
                 } else {
-                    group_scatter<F, MEM>(m, cache, lists, cnt, b, ordered, -1, t, 32);
+                    group_scatter<F, MEM>(m, cache, lists, cnt, b, t, 32);
                     __syncwarp();
                 }
             }
@@ -787,7 +858,7 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
                 const int cnt = ctl[4 + 2 * acc.par], own = ctl[5 + 2 * acc.par];
                 acc.par ^= 1;
                 if (cnt < 0) break;
-                group_scatter<F, MEM>(m, cache, lists, cnt, own, ordered, bar_id, t, tpr);
+                group_scatter<F, MEM>(m, cache, lists, cnt, own, t, tpr);
                 named_bar(bar_id, tpr);
             }
         }

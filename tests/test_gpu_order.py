@@ -31,9 +31,9 @@ def test_tracked_energies_of_narrow_levels():
     """Per-sweep energies of an fp32 model with levels of about 13 variables.
     Couplings and values are whole numbers, so fields and energy changes are exact
     and both orders make the same moves; what is left is the rounding of the sums
-    of changes.  It falls with the root of the number of partial sums (32 lanes of
-    a block against the threads of a level), so blocks may be no worse than half as
-    much again as levels."""
+    of changes, if any.  It falls with the root of the number of partial sums (32
+    lanes of a block against the threads of a level), so blocks may be no worse than
+    half as much again as levels."""
     n, S, R = 1000, 4, 64
     inst = wl.quio_sparse_int(4, n, 20 * n, 0, 200)
     inst = dict(inst, coeffs=inst["coeffs"].astype(np.float32), coef_type="f32")
@@ -52,5 +52,86 @@ def test_tracked_energies_of_narrow_levels():
         assert torch.equal(ta, tb)
         true = torch.stack([model.energy(ta[s]) for s in range(S)])
         rms = [float(((e - true)[:-1] ** 2).mean().sqrt()) for e in (ea, eb)]
-        assert rms[1] > 0 and rms[0] <= 1.5 * rms[1], (rule, rms)
+        assert rms[0] <= 1.5 * rms[1], (rule, rms)
         assert torch.equal(ea[-1], true[-1])     # recomputed in FP64 at the end, whole numbers
+
+
+def _gaussian(n, deg, lo, hi, path=False, seed=6):
+    """Sparse fp32 model with Gaussian couplings (sums depend on their order);
+    `path` couples neighbours too, so that every level holds one variable."""
+    rng = np.random.default_rng(seed)
+    full = deg >= n - 1
+    pairs = [(i, j) for i in range(n) for j in range(i + 1, n)] if full else None
+    if full:      # all couplings but one
+        pairs = [p for p in pairs if p != (0, n - 1)]
+    else:
+        keep = rng.random((n, n)) < deg / n
+        pairs = [(i, j) for i in range(n) for j in range(i + 1, n) if keep[i, j] or (path and j == i + 1)]
+    pairs = np.array(pairs)
+    offs = np.concatenate([np.arange(n + 1), n + 2 * np.arange(1, n + 1),
+                           3 * n + 2 * np.arange(1, len(pairs) + 1)]).astype(np.int64)
+    flat = np.concatenate([np.arange(n), np.repeat(np.arange(n), 2), pairs.ravel()]).astype(np.int32)
+    c = np.concatenate([rng.normal(size=n), rng.random(n), rng.normal(size=len(pairs))]).astype(np.float32)
+    return {"n_vars": n, "lower": np.full(n, lo, np.int64), "upper": np.full(n, hi, np.int64), "term_offsets": offs,
+            "term_vars": flat, "coeffs": c, "coef_type": "f32"}
+
+
+# (variables, degree, bounds, neighbours coupled): rows of one piece of 32 links
+# and of several, columns split over several warps, ragged last blocks, one block,
+# a complete graph without one coupling, rows that almost fill their columns
+ORDER_CASES = {
+    "short_rows": (300, 20, 0, 40, False), "two_pieces": (500, 60, -5, 9, False), "long_rows": (700, 330, 0, 3, False),
+    "one_block": (31, 12, 0, 20, False), "edge_33": (33, 16, -9, 9, False), "wide": (260, 40, 0, 300, False),
+    "all_but_one": (421, 421, -4, 4, False), "all_but_one_65": (65, 65, 0, 90, False),
+    "path_short": (300, 12, 0, 30, True), "path_long": (640, 200, -6, 6, True), "path_hub": (97, 60, 0, 2, True),
+}
+
+
+@pytest.mark.parametrize("case", sorted(ORDER_CASES))
+@pytest.mark.parametrize("rule", RULES)
+def test_fp32_runs_do_not_depend_on_their_threads(case, rule):
+    """Blocked runs: the same bits for every thread count, in shared and global
+    memory, plain and time-sliced, batched and served."""
+    from paper_2511_17245_gb300 import (make_params, sa_batch_create, sa_batch_destroy, sa_batch_result, sa_batch_run,
+                                        sa_server_create, sa_server_destroy, sa_server_result, sa_server_submit,
+                                        sa_server_wait)
+    n, deg, lo, hi, path = ORDER_CASES[case]
+    model = Model(_gaussian(n, deg, lo, hi, path))
+    levels = model.info["n_levels"]
+    assert levels * (3 if rule == "heat_bath" else 16) >= n or rule == "heat_bath"
+    if levels * 3 < n and rule == "heat_bath":
+        pytest.skip("the heat bath keeps the level order here")
+    S, R = 60, 20
+    # (the heat bath's form of a sum follows the thread count, see sa.h: one count there)
+    counts = (32, 64, 128, 256, 512) if rule != "heat_bath" else (128,)
+    runs = {f"threads {t}": model.run(rule, S, R, seed=2, threads_per_replica=t) for t in counts}
+    runs["global"] = model.run(rule, S, R, seed=2, threads_per_replica=counts[-1], flags=_lib.SA_FLAG_STATE_IN_GLOBAL)
+    ref = runs[f"threads {counts[0]}"]
+    for name, got in runs.items():
+        assert torch.equal(ref["states"], got["states"]), name
+        assert torch.equal(ref["accepts"], got["accepts"]), name
+    if path or case.startswith("all_but_one"):   # one variable per level: the level order's bits too
+        lvl = model.run(rule, S, R, seed=2, threads_per_replica=counts[0], flags=_lib.SA_FLAG_NO_SPECULATION)
+        if levels == n:
+            for key in ("states", "accepts", "energies"):
+                assert torch.equal(ref[key], lvl[key]), key
+    if rule == "heat_bath":
+        return
+    many = model.run(rule, S, 700, seed=2, threads_per_replica=256)["states"]
+    plain = model.run(rule, S, 700, seed=2, threads_per_replica=256, flags=_lib.SA_FLAG_NO_TIME_SLICING)["states"]
+    assert torch.equal(many, plain) and torch.equal(many[:R], ref["states"])
+    p = make_params(rule=rule, n_sweeps=S, n_replicas=R, seed=2)
+    st = [np.zeros((R, n), np.int32) for _ in range(2)]
+    en, ac = np.zeros(R), np.zeros(R, np.uint64)
+    b = sa_batch_create([model.handle], [p])
+    sa_batch_run(b)
+    torch.cuda.synchronize()
+    sa_batch_result(b, 0, st[0], en, ac)
+    sa_batch_destroy(b)
+    srv = sa_server_create(budget_bytes=1 << 28, max_running=4)
+    ticket = sa_server_submit(srv, model.handle, p)
+    sa_server_wait(srv, ticket, 60_000_000)
+    sa_server_result(srv, ticket, st[1], en, ac)
+    sa_server_destroy(srv)
+    for s in st:
+        assert np.array_equal(s, ref["states"].cpu().numpy())
