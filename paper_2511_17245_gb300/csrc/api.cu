@@ -459,9 +459,13 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         for (auto& t : terms)
             for (auto& m : t.mem) omega[m.var] |= (1ull << m.exp);
         std::vector<int32_t> slot_base(n + 1, 0);
-        // (multilinear models: one slot per variable, used or not, so that slot = variable)
+        // (multilinear models of which few variables are unused: one slot per
+        // variable, so that slot = variable; a replica's region is no larger for it)
+        int64_t unused = 0;
+        for (int32_t k = 0; k < n; ++k) unused += omega[k] == 0;
+        const bool slot_per_var = multilinear && unused * (M->is_float ? 4 : 8) <= sa::kSlotSlack;
         for (int32_t k = 0; k < n; ++k)
-            slot_base[k + 1] = slot_base[k] + (multilinear ? 1 : __builtin_popcountll(omega[k]));
+            slot_base[k + 1] = slot_base[k] + (slot_per_var ? 1 : __builtin_popcountll(omega[k]));
         const int32_t n_slots = slot_base[n];
         auto slot_of = [&](int32_t k, int32_t e) {
             return slot_base[k] + __builtin_popcountll((omega[k] & ((1ull << e) - 1ull)) >> 1);
@@ -542,7 +546,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
                 q[3] = packed;
             }
         // the compact form (DevModel::inc16)
-        bool compact = multilinear && n <= 65534 && max_order <= 4 && dm.z_span <= (uint32_t)INT32_MAX;
+        bool compact = slot_per_var && n <= 65534 && max_order <= 4 && dm.z_span <= (uint32_t)INT32_MAX;
         for (int32_t k = 0; k < n && compact; ++k) compact = lo[k] == dm.z_base;
         if (!M->is_float)
             for (int32_t tt = 0; tt < n_iterms && compact; ++tt) compact = tcoef_i[tt] == (int64_t)(int32_t)tcoef_i[tt];

@@ -93,9 +93,9 @@ struct DevModel {
     // {their variables v1..v3, term}, {their coefficient slots (slot_base[v] +
     // index of the exponent), 0}, {their lower bounds, 0}
     const int32_t* inc_rec;
-    // multilinear models of at most 65,534 variables with one lower bound, terms
-    // of at most 4 members and coefficients that fit 32 bits: the same in one
-    // 16-byte group, {coefficient (int32 or fp32 bits), v1 | v2 << 16, v3, 0} with
+    // multilinear models of at most 65,534 variables, few of them in no term, with
+    // one lower bound, terms of at most 4 members and coefficients that fit 32
+    // bits: the same in one 16-byte group, {coefficient (int32 or fp32 bits), v1 | v2 << 16, v3, 0} with
     // 0xFFFF for no variable (variable v's slot is v); null otherwise
     const int32_t* inc16;
     const int32_t* term_ptr;    // [n_iterms + 1] into mem_var / mem_exp
@@ -340,7 +340,7 @@ struct RunPlan {
     int32_t rpc;                // replicas per block
     int32_t blocks;
     int32_t heavy_links;        // update lists above this length go to the cooperative list
-    int32_t list_cap;           // entries of the cooperative list (6 ints each)
+    int32_t list_cap;           // entries of the cooperative list (list_words each)
     int32_t in_global;          // replica state in global memory instead of shared memory
     int64_t rep_bytes;          // bytes of one replica's state region
     int64_t shared_bytes;       // dynamic shared memory of one block
@@ -349,6 +349,13 @@ struct RunPlan {
 };
 
 inline int64_t plan_round16(int64_t x) { return (x + 15) / 16 * 16; }
+
+// Words of an entry of the cooperative list (five are used; QUIO's lists hold a
+// blocked sweep's two lists of 32 16-byte commits as well).
+constexpr int list_words(int kind) { return kind == KIND_HUIO ? 5 : 6; }
+// Bytes that the shorter entries save in the region of a HUIO replica, for slots
+// of unused variables (see compile_terms).
+constexpr int64_t kSlotSlack = 256 * 4;
 
 // State layout of one replica for `tpr` threads: offsets z_k - l_k (zbytes
 // each), the cache (int64 or fp32), the control words (three list counters or
@@ -369,7 +376,7 @@ inline int64_t plan_layout(const PlanModel& m, int zbytes, int tpr, RunPlan* p) 
     p->off_cache = (int32_t)plan_round16((int64_t)m.n * zbytes);
     p->off_ctl = (int32_t)plan_round16(p->off_cache + m.cache_elems * fsize);
     p->off_list = p->off_ctl + 112;
-    p->off_red = (int32_t)plan_round16(p->off_list + (int64_t)p->list_cap * 24);
+    p->off_red = (int32_t)plan_round16(p->off_list + (int64_t)p->list_cap * list_words(m.kind) * 4);
     const int64_t lvl_bytes = (int64_t)(m.n_levels + 1) * 4;
     const int64_t off_lvl = plan_round16(p->off_red + (int64_t)(tpr / 32) * 8);
     const bool lvl_on_chip = lvl_bytes <= 16384;

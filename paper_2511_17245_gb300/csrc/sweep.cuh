@@ -1385,16 +1385,17 @@ __device__ __forceinline__ void solo_add(float* c, float w, long long dz) {
 __device__ __forceinline__ void solo_add(long long* c, long long w, long long dz) { *c += w * dz; }
 
 // ------------------------------------------------------------------ shared update lists
-// The list of a level's accepted variables ([nl][6]: variable, z_old, z_new,
-// first link, links) flattened into (entry, link) pairs.  Every warp forms the
-// prefix of 32 entries' lengths by itself and its lanes find their entries by
-// bisection over the warp.
+// The list of a level's accepted variables (list_words(KIND) words each: variable,
+// z_old, z_new, first link, links) flattened into (entry, link) pairs.  Every warp
+// forms the prefix of 32 entries' lengths by itself and its lanes find their
+// entries by bisection over the warp.
 struct ListChunk {
     int len, inc, total;   // this lane's entry's links, their inclusive prefix, the chunk's links
 };
+template <int KIND>
 __device__ __forceinline__ ListChunk list_chunk(const int* list, int h0, int nl, int lane) {
     ListChunk q;
-    q.len = h0 + lane < nl ? list[6 * (h0 + lane) + 4] : 0;
+    q.len = h0 + lane < nl ? list[list_words(KIND) * (h0 + lane) + 4] : 0;
     q.inc = q.len;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1405,13 +1406,14 @@ __device__ __forceinline__ ListChunk list_chunk(const int* list, int h0, int nl,
     return q;
 }
 // Link of the chunk's pair w (-1 beyond the last) and its entry.
+template <int KIND>
 __device__ __forceinline__ int list_find(const ListChunk& q, const int* list, int h0, int w, const int*& ent) {
     int h = 0;   // number of entries that end at or before w
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
         if (__shfl_sync(0xffffffffu, q.inc, h + o - 1) <= w) h += o;
     const int pre = __shfl_sync(0xffffffffu, q.inc - q.len, h);
-    ent = list + 6 * (h0 + h);
+    ent = list + list_words(KIND) * (h0 + h);
     return w < q.total ? ent[3] + (w - pre) : -1;
 }
 
@@ -1427,7 +1429,7 @@ __device__ __noinline__ void huio_group_update(const DevModel& m, const Z* zs_an
     const int4* inc16 = reinterpret_cast<const int4*>(m.inc16);
     const int z_base = m.z_base;
     for (int h0 = 0; h0 < nl; h0 += 32) {
-        const ListChunk c = list_chunk(list, h0, nl, lane);
+        const ListChunk c = list_chunk<KIND_HUIO>(list, h0, nl, lane);
         if (inc16 != nullptr) {
             for (int w0 = t - lane; w0 < c.total; w0 += 4 * tpr) {
                 int dz[4];
@@ -1438,7 +1440,7 @@ __device__ __noinline__ void huio_group_update(const DevModel& m, const Z* zs_an
                     on[u] = false;
                     if (w0 + u * tpr < c.total) {
                         const int* ent;
-                        const int e = list_find(c, list, h0, w0 + u * tpr + lane, ent);
+                        const int e = list_find<KIND_HUIO>(c, list, h0, w0 + u * tpr + lane, ent);
                         on[u] = e >= 0;
                         if (on[u]) {
                             q[u] = __ldg(inc16 + e);
@@ -1453,8 +1455,8 @@ __device__ __noinline__ void huio_group_update(const DevModel& m, const Z* zs_an
         } else {
             for (int w0 = t - lane; w0 < c.total; w0 += 2 * tpr) {
                 const int *ea, *eb;
-                const int la = list_find(c, list, h0, w0 + lane, ea);
-                const int lb = w0 + tpr < c.total ? list_find(c, list, h0, w0 + tpr + lane, eb) : -1;
+                const int la = list_find<KIND_HUIO>(c, list, h0, w0 + lane, ea);
+                const int lb = w0 + tpr < c.total ? list_find<KIND_HUIO>(c, list, h0, w0 + tpr + lane, eb) : -1;
                 IncRec qa, qb;
                 if (la >= 0) qa = load_inc(m, la);
                 if (lb >= 0) qb = load_inc(m, lb);
@@ -1471,11 +1473,11 @@ __device__ __forceinline__ void quio_group_update(const DevModel& m, F* cache, c
                                                   bool solo) {
     const int lane = t & 31;
     for (int h0 = 0; h0 < nl; h0 += 32) {
-        const ListChunk c = list_chunk(list, h0, nl, lane);
+        const ListChunk c = list_chunk<KIND_QUIO>(list, h0, nl, lane);
         for (int w0 = t - lane; w0 < c.total; w0 += 2 * tpr) {
             const int *ea, *eb;
-            const int la = list_find(c, list, h0, w0 + lane, ea);
-            const int lb = w0 + tpr < c.total ? list_find(c, list, h0, w0 + tpr + lane, eb) : -1;
+            const int la = list_find<KIND_QUIO>(c, list, h0, w0 + lane, ea);
+            const int lb = w0 + tpr < c.total ? list_find<KIND_QUIO>(c, list, h0, w0 + tpr + lane, eb) : -1;
             int ca = 0, cb = 0;
             F wa = F(0), wb = F(0);
             if (la >= 0) { ca = __ldg(m.adj_col + la); wa = Coef<F>::adj(m, la); }
@@ -1601,8 +1603,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
     F* cache = reinterpret_cast<F*>(base + a.off_cache);
     // [0..2] list counters; blocked sweeps: [0..1] commits of the two lists, [4..7] commands
     int* ctl = reinterpret_cast<int*>(base + a.off_ctl);
-    // [cap][6]: variable k, z_old, z_new, link_begin, link_len, prefix of the
-    // flattened (entry, link) pairs
+    // [cap][list_words(KIND)]: variable k, z_old, z_new, link_begin, link_len
     int* list = reinterpret_cast<int*>(base + a.off_list);
     Acc* red = reinterpret_cast<Acc*>(base + a.off_red);
 
@@ -1739,7 +1740,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
             if (!inline_upd) {
                 const int idx = atomicAdd(cnt_now, 1);
                 if (idx < a.list_cap) {
-                    int* e = list + 6 * idx;
+                    int* e = list + list_words(KIND) * idx;
                     e[0] = k;
                     e[1] = (int)z;
                     e[2] = (int)v;

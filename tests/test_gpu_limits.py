@@ -10,7 +10,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from paper_2511_17245_gb300 import (Model, make_params, sa_batch_create, sa_batch_destroy, sa_batch_get_info,
+from paper_2511_17245_gb300 import (Model, _lib, make_params, sa_batch_create, sa_batch_destroy, sa_batch_get_info,
                                     sa_batch_result, sa_batch_run)
 from paper_2511_17245_gb300 import workloads as wl
 
@@ -78,3 +78,30 @@ assert np.array_equal(got, want), (got, want)
 """
     res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, res.stderr[-2000:]
+
+
+@pytest.mark.parametrize("n,first", [(20_000, 0), (20_000, 19_000), (188, 0), (188, 9), (189, 3)])
+def test_unused_variables_take_no_coefficient_slots(n, first):
+    """A multilinear HUIO model, 60 of whose variables occur in terms: 100 replicas
+    of 20,000 variables take 2.7 MB of the fixed scratch of sa_run_noalloc, not 18.
+    With 128 unused variables the slots are padded, with 129 they are not."""
+    from oracle import oracle as orc
+    from paper_2511_17245_gb300 import sa_run_noalloc
+    small = wl.random_small(3, 60, 4, np.full(60, -3), np.full(60, 4), 300, repeat=False)
+    used = first + 3 * np.arange(60)
+    inst = dict(small, n_vars=n, lower=np.full(n, -3, np.int64), upper=np.full(n, 4, np.int64),
+                term_vars=used[small["term_vars"]].astype(np.int32))
+    model, om = Model(inst), orc.Model(inst)
+    R, S = 100, 12
+    tmax, tmin = om.auto_temperatures()
+    st = torch.empty((R, n), dtype=torch.int32, device="cuda")
+    en = torch.empty(R, dtype=torch.int64, device="cuda")
+    tr = torch.zeros((S, 3, n), dtype=torch.int32, device="cuda")
+    sa_run_noalloc(model.handle, make_params(rule="metropolis", n_sweeps=S, n_replicas=R, seed=4, t_max=tmax,
+                                             t_min=tmin, flags=_lib.SA_FLAG_STATE_IN_GLOBAL, trace=tr,
+                                             trace_replicas=3), st, en)
+    torch.cuda.synchronize()
+    res = om.run("metropolis", S, 4, tmax, tmin, r_begin=0, r_end=3, trace=tr.cpu().numpy(), trace_replicas=3)
+    assert res["follow"]["mismatch"] == 0, res["follow"]
+    assert np.array_equal(res["states"], st[:3].cpu().numpy())
+    assert torch.equal(en, model.energy(st))
