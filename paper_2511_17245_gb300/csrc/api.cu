@@ -600,8 +600,8 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         off.omega = blob.add(omega);
         off.inc_term = blob.add(inc_term);
         off.inc_exp = blob.add(inc_exp);
-        off.inc_rec = blob.add(inc_rec);
-        if (compact) off.inc16 = blob.add(inc16);
+        if (compact) off.inc16 = blob.add(inc16);   // (the sweeps read one form or the other)
+        else off.inc_rec = blob.add(inc_rec);
         off.term_ptr = blob.add(term_ptr);
         off.mem_var = blob.add(mem_var);
         off.mem_exp = blob.add(mem_exp);
@@ -655,7 +655,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
         dm.omega = at<uint64_t>(b, off.omega);
         dm.inc_term = at<int32_t>(b, off.inc_term);
         dm.inc_exp = at<int32_t>(b, off.inc_exp);
-        dm.inc_rec = at<int32_t>(b, off.inc_rec);
+        dm.inc_rec = off.inc16 == SIZE_MAX ? at<int32_t>(b, off.inc_rec) : nullptr;
         dm.inc16 = off.inc16 == SIZE_MAX ? nullptr : at<int32_t>(b, off.inc16);
         dm.term_ptr = at<int32_t>(b, off.term_ptr);
         dm.mem_var = at<int32_t>(b, off.mem_var);

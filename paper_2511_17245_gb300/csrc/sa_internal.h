@@ -91,7 +91,7 @@ struct DevModel {
     // 1 << 16 when every exponent is 1 (or -1 for terms of more than 4
     // members), the other members' exponents packed e1 | e2 << 8 | e3 << 16},
     // {their variables v1..v3, term}, {their coefficient slots (slot_base[v] +
-    // index of the exponent), 0}, {their lower bounds, 0}
+    // index of the exponent), 0}, {their lower bounds, 0}; null where inc16 is not
     const int32_t* inc_rec;
     // multilinear models of at most 65,534 variables, few of them in no term, with
     // one lower bound, terms of at most 4 members and coefficients that fit 32

@@ -105,3 +105,39 @@ def test_unused_variables_take_no_coefficient_slots(n, first):
     assert res["follow"]["mismatch"] == 0, res["follow"]
     assert np.array_equal(res["states"], st[:3].cpu().numpy())
     assert torch.equal(en, model.energy(st))
+
+
+@pytest.mark.parametrize("lows", [(-2,), (-2, -1)])
+def test_levels_with_more_changes_than_list_places(lows):
+    """Levels of more than 256 variables that nearly all change: the lists that find
+    no place are walked by their lanes, from compact records (one lower bound) and
+    full ones (two), to the oracle's states."""
+    from oracle import oracle as orc
+    n, S, R = 1800, 4, 3
+    rng = np.random.default_rng(8)
+    lo = np.resize(np.asarray(lows), n)
+    terms = [[k] for k in range(n)] + [sorted(rng.choice(n, 1 + int(rng.integers(1, 4)), replace=False))
+                                       for _ in range(n // 2)]
+    offs = np.concatenate([[0], np.cumsum([len(t) for t in terms])]).astype(np.int64)
+    inst = {"n_vars": n, "lower": lo.astype(np.int64), "upper": (lo + 9).astype(np.int64), "term_offsets": offs,
+            "term_vars": np.concatenate(terms).astype(np.int32),
+            "coeffs": rng.integers(1, 6, len(terms)).astype(np.int32), "coef_type": "i32"}
+    model, om = Model(inst), orc.Model(inst)
+    later = {int(v) for t in terms for v in t[1:]}   # (members after a term's first have an earlier neighbour)
+    assert n - len(later) > 512                      # variables of the first level
+    for rule in ("metropolis", "opt_metropolis"):
+        tr = torch.zeros((S, R, n), dtype=torch.int32, device="cuda")
+        out = model.run(rule, S, R, seed=3, t_max=1e6, t_min=1e5, trace=tr, trace_replicas=R)
+        res = om.run(rule, S, 3, 1e6, 1e5, r_begin=0, r_end=R, trace=tr.cpu().numpy(), trace_replicas=R)
+        assert res["follow"]["mismatch"] == 0, res["follow"]
+        assert np.array_equal(res["states"], out["states"].cpu().numpy())
+        assert np.array_equal(res["energy"], out["energies"].cpu().numpy())
+
+
+def test_a_model_holds_one_record_per_incidence():
+    """Compact records: 16 bytes an incidence beside the term lists' 16 and 8 per
+    term (at least two incidences); with full records it was 100 and more."""
+    inst = wl.huio_zipf(1, n=2000, n_quad=8000, n_cubic=20_000, n_quartic=5000)
+    lens = np.diff(inst["term_offsets"])
+    incidences = int(lens[lens > 1].sum())
+    assert Model(inst).info["device_bytes"] <= 36 * incidences + 200 * 2000 + (1 << 16)
