@@ -214,13 +214,15 @@ typedef struct {
  * sequential trajectory exactly for integer models.
  *
  * Blocked sweeps (QUIO): models whose levels are narrow (up to 16 variables on
- * average, up to 3 for the heat bath; every level of a complete graph holds
- * one) are swept in blocks of 32 consecutive variables, decided by one warp at
- * once.  A decision is kept when no earlier variable of the block that shares a
+ * average; for the heat bath up to 3, 1.1 where ranges are wide; every level of a
+ * complete graph holds one) are swept in blocks of 32 consecutive variables,
+ * decided by one warp at once.  A decision is kept when no earlier variable of the block that shares a
  * term with it changes in the same round; the others are made again with the
  * changes in their fields.  States, counts and traces are those of the
  * level-by-level order, bit for bit (float models included where every level
- * holds one variable, and energies too at the same thread count).
+ * holds one variable, and energies too at the same thread count).  Float fields
+ * take their changes in the visiting order, so that the states of a Metropolis
+ * run do not depend on the threads or on the form of its launch.
  * SA_FLAG_NO_SPECULATION keeps the level-by-level order.
  *
  * Time slicing: when the replicas' state stays in shared memory but more

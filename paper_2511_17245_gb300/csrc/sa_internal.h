@@ -271,21 +271,41 @@ struct PlanModel {
     int32_t block_model;        // the model holds the tables of the blocked sweep
     int32_t dense_rows;         // complete graph
     int32_t mean_links;         // mean length of the neighbour lists
+    uint32_t max_width;         // largest u_k - l_k
 };
 
 inline PlanModel plan_model(const ModelView& v) {
     return PlanModel{v.n, v.n_levels, v.dm.kind, v.is_float, v.zbytes, v.max_link_len, v.cache_elems,
-                     v.dm.idx_rec != nullptr, v.dm.dense_rows, (int32_t)(v.n_links / (v.n > 0 ? v.n : 1))};
+                     v.dm.idx_rec != nullptr, v.dm.dense_rows, (int32_t)(v.n_links / (v.n > 0 ? v.n : 1)),
+                     v.dm.max_width};
 }
 
 // ------------------------------------------------------------------ blocked sweeps
 // A level costs a group barrier, a Philox block and an L2 round trip whatever
 // its width; a block of 32 variables costs one of each plus a short round per
-// colliding change.  kBlockWidth is the mean level width up to which blocks win
-// (QUIO), kBlockWidthHeat the same for the heat bath, whose decisions a block
-// makes one after the other and a level side by side.
+// colliding change.  kBlockWidth is the mean level width up to which models hold
+// the tables of the blocked sweep (QUIO) and the Metropolis rules use it: 1000
+// variables, 64 replicas x 20 sweeps, blocks against levels 0.66 against 1.96 ms
+// at a width of 7, 2.0 against 4.5 at 13, 2.1 against 5.6 at 15; 1024 replicas
+// 3.4 against 4.8 and 5.8 there.
 constexpr int kBlockWidth = 16;
-constexpr int kBlockWidthHeat = 3;
+
+// The heat bath's limit, by the number of values of the widest range.  A block
+// decides wide ranges one variable after the other by one warp, a level side by
+// side by all of them, so the limit falls as a decision grows.  Times in ms of 5
+// sweeps, 64 / 1024 replicas, blocks against levels (1000 variables, * 200):
+//   fp32    64 values: width 2.3   5.6 / 11.5 against 6.2 / 14.1; * 2.7  1.08 / 1.44 against 0.95 / 1.32
+//          128 values: width 2.3   6.9 / 13.0 against 6.4 / 14.6; * 2.7  1.29 / 1.64 against 1.03 / 1.40
+//          256 values: width 1.7  11.2 / 20.0 against 10.5 / 22.5;  2.3  10.8 / 15.8 against 7.8 / 16.2
+//         1024 values: width 1.3  15.3 / 29.1 against 16.3 / 33.2;  1.7  14.6 / 25.4 against 12.6 / 26.3
+//   int64   48 values: * 2.7  2.4 / 3.1 against 3.0 / 3.9 (wide levels begin at 57)
+//          256 values: width 1.4  13.3 / 28.4 against 13.7 / 27.3;  1.8  12.7 / 23.9 against 10.9 / 21.9
+//         1024 values: width 1.1  21.2 / 42.4 against 23.8 / 44.1; * 1.2  4.1 / 5.8 against 4.3 / 5.8
+inline double block_width_heat(bool is_float, uint32_t max_width) {
+    const int64_t values = (int64_t)max_width + 1;
+    if (is_float) return values <= 128 ? 2.5 : (values <= 256 ? 1.75 : 1.5);
+    return values <= 56 ? 3.0 : (values <= 256 ? 1.5 : 1.1);
+}
 
 inline bool plan_block_model(int32_t n, int32_t n_levels) { return (int64_t)n <= (int64_t)kBlockWidth * n_levels; }
 
@@ -293,7 +313,7 @@ inline bool plan_block_model(int32_t n, int32_t n_levels) { return (int64_t)n <=
 // ask for the level order).
 inline bool plan_blocked(const PlanModel& m, int rule, bool allowed) {
     if (!m.block_model || !allowed) return false;
-    return rule != RULE_HEAT_BATH || (int64_t)m.n <= (int64_t)kBlockWidthHeat * m.n_levels;
+    return rule != RULE_HEAT_BATH || (double)m.n <= block_width_heat(m.is_float != 0, m.max_width) * (double)m.n_levels;
 }
 
 // Whether the model holds the pair list that the energies of states are summed

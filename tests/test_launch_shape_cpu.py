@@ -200,3 +200,23 @@ def test_batch_shapes_count_the_argument_copies(tmp_path):
 """
     bad, seen, rem = (int(x) for x in _compile_and_run(tmp_path, body))
     assert bad == 0 and rem == 0 and seen > 400_000
+
+
+@pytest.mark.parametrize("n,levels,is_float,width,want", [
+    (1000, 1000, 0, 4000, 1), (1000, 909, 0, 1023, 0), (1000, 910, 0, 1023, 1),      # int64, wide: 1.1
+    (1000, 666, 0, 255, 0), (1000, 667, 0, 255, 1), (1000, 667, 0, 256, 0),          # up to 256 values: 1.5
+    (1000, 333, 0, 55, 0), (999, 333, 0, 55, 1), (999, 333, 0, 56, 0),               # up to 56 values: 3
+    (1000, 400, 1, 127, 1), (1000, 399, 1, 127, 0), (1000, 400, 1, 128, 0),          # fp32, up to 128: 2.5
+    (1001, 572, 1, 255, 1), (1001, 571, 1, 255, 0),                                  # up to 256: 1.75
+    (999, 666, 1, 256, 1), (1000, 666, 1, 256, 0),                                   # wider: 1.5
+])
+def test_heat_bath_takes_blocks_where_levels_are_narrow_for_its_ranges(tmp_path, n, levels, is_float, width, want):
+    """A block decides wide ranges in turn by one warp, a level side by side: the
+    limit of the level width falls with the range.  Other rules do not look at it."""
+    body = f"""
+  sa::PlanModel m{{{n}, {levels}, sa::KIND_QUIO, {is_float}, 2, 40, {n}, 1, 0, 40, {width}u}};
+  std::printf("%d %d %d %d\\n", (int)sa::plan_blocked(m, sa::RULE_HEAT_BATH, true),
+              (int)sa::plan_blocked(m, sa::RULE_HEAT_BATH, false), (int)sa::plan_blocked(m, sa::RULE_METROPOLIS, true),
+              (int)sa::plan_blocked(m, sa::RULE_OPT, true));
+"""
+    assert [int(x) for x in _compile_and_run(tmp_path, body)] == [want, 0, 1, 1]
