@@ -266,7 +266,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
     dm.const_i = (int64_t)const_i;
     dm.const_d = const_d;
     struct Offs {
-        size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk_w = 0, blk_i = 0;
+        size_t meta, lvl_ptr, lvl_vars, lvl_rec, idx_rec = 0, blk_mask = 0, blk_w = 0, blk_i = 0, blk_part = 0;
         bool blk_wide = false;
         size_t up_rec, up_pair = SIZE_MAX, adj_col, adj_i, adj_f, adj_d, lin_i, lin_f, lin_d, diag_i, diag_f, diag_d;
         size_t slot_base, omega, aconst_i, aconst_f, aconst_d, inc_term, inc_exp, inc_rec, inc16 = SIZE_MAX, term_ptr, mem_var, mem_exp,
@@ -439,6 +439,16 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
             off.blk_mask = blob.add(mask);
             off.blk_w = blob.add(bw);
             if (off.blk_wide) off.blk_i = blob.add(bi);
+            if (M->is_float && !dm.dense_rows) {
+                const int32_t per = sa::plan_row_part(n);
+                std::vector<int32_t> part((size_t)n * sa::kRowParts);
+                for (int32_t k = 0; k < n; ++k)
+                    for (int64_t p = 0; p < sa::kRowParts; ++p)
+                        part[(size_t)k * sa::kRowParts + p] =
+                            (int32_t)(std::lower_bound(col.begin() + ptr[k], col.begin() + ptr[k] + deg[k], p * per) -
+                                      (col.begin() + ptr[k]));
+                off.blk_part = blob.add(part);
+            }
         }
         if (M->is_float) {
             std::vector<float> vf(vd.size()), lf(n), df(n);
@@ -637,6 +647,7 @@ sa_status compile_terms(sa_model* M, int32_t n, const int64_t* lower, const int6
             dm.blk_mask = at<uint32_t>(b, off.blk_mask);
             dm.blk_w = at<int32_t>(b, off.blk_w);
             if (off.blk_wide) dm.blk_i = at<int64_t>(b, off.blk_i);
+            if (M->is_float && !dm.dense_rows) dm.blk_part = at<int32_t>(b, off.blk_part);
         }
         dm.adj_col = at<int32_t>(b, off.adj_col);
         dm.up_rec = at<int32_t>(b, off.up_rec);

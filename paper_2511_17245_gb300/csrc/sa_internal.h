@@ -51,6 +51,8 @@ struct DevModel {
     const LevelRec* idx_rec;    // [n]: records in index order, slot_base = width of the variable's level
     const uint32_t* blk_mask;   // [n]: bit j set iff variable 32 (k / 32) + j < k shares a term with k
     const int32_t* blk_w;       // [32 ceil(n / 32)][32]: J_kj of the variables j of k's block (fp32 bits or int32)
+    const int32_t* blk_part;    // fp32 models [n][kRowParts]: first entry of row k, from the row's start, whose
+                                // column is in part p of the columns or a later one (plan_row_part)
     const int64_t* blk_i;       // the same in int64, when some J_kj does not fit int32 (blk_w is not read then)
 
     // QUIO (every term of total degree <= 2):
@@ -323,6 +325,11 @@ inline bool plan_blocked(const PlanModel& m, int rule, bool allowed) {
 inline bool plan_pair_list(int32_t n, int64_t lo, int64_t hi, int64_t pairs) {
     return n <= 65536 && lo > -4096 && hi < 4096 && pairs <= 32 * (int64_t)n;
 }
+
+// Parts of the columns (whole blocks of 32) that the warps of a group take when
+// they add a block's changes to fp32 fields in order; columns of one part.
+constexpr int kRowParts = 16;
+inline int32_t plan_row_part(int32_t n) { return ((n + 31) / 32 + kRowParts - 1) / kRowParts * 32; }
 
 // Bytes of one block staged on chip: couplings (32 x 32 x 4), records, masks.
 constexpr int kBlockStage = 4096 + 32 * (int)sizeof(LevelRec) + 128;

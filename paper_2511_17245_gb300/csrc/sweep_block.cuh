@@ -352,10 +352,16 @@ __device__ __noinline__ void scatter_commits(const DevModel& m, F* cache_any, co
 
 // fp32 fields of any graph: every field takes its changes in the order of the
 // commits, so that a run's results do not depend on its threads.  Each of `nw`
-// warps owns a range of columns and walks the commits over its part of their rows
-// (rows are sorted by column), 32 links at a time with plain reads and writes;
-// eight such pieces are loaded before the first is added.
-// What bounds it: a shared-memory round trip per piece and an L2 one per eight.
+// warps (a power of two) owns a range of columns and walks the commits over its
+// part of their rows (rows are sorted by column, DevModel::blk_part holds where the
+// parts begin), 32 links at a time with plain reads and writes; eight such pieces
+// are loaded before the first is added.
+// What bounds it: the instructions of a piece (about 25) and its shared-memory
+// round trip, one warp's chain; sixteen pieces at a time or the next eight loaded
+// ahead cost more in pieces past the last.  1000 variables, Metropolis, 64 / 1024
+// replicas x 20 sweeps, unordered atomics over all threads against this: rows of 40
+// links 2.01 / 3.45 ms against 2.26 / 3.17, 120 links 2.26 / 6.65 against 2.55 /
+// 5.17, 500 links 4.54 / 22.5 against 4.26 / 15.0.
 template <int MEM>
 __device__ __noinline__ void ordered_commits(const DevModel& m, float* cache_any, const Commit* list_any, int count,
                                              int own, int warp, int nw, int lane) {
@@ -363,25 +369,16 @@ __device__ __noinline__ void ordered_commits(const DevModel& m, float* cache_any
     constexpr int U = 8;
     float* cache = in_shared<MEM>(cache_any);
     const Commit* list = in_shared<MEM>(list_any);
-    // lane c: commit c's part of this warp's columns, [row + first, row + last)
-    const Commit e = list[lane];   // (entries beyond the count are read and not used)
-    const int row = e.z;
-    int first = 0, last = lane < count ? e.w : 0;
-    if (nw > 1) {
-        const int per = (((m.n + 31) >> 5) + nw - 1) / nw * 32;
-        // the row's first entry whose column is c or above; columns are distinct,
-        // which leaves few candidates in a nearly full row
-        auto find = [&](int c) -> int {
-            int a = max(0, last - max(0, m.n - c)), b = min(last, c);
-            while (a < b) {
-                const int mid = (a + b) >> 1;
-                if (__ldg(m.adj_col + row + mid) < c) a = mid + 1;
-                else b = mid;
-            }
-            return a;
-        };
-        first = find(warp * per);
-        last = find((warp + 1) * per);
+    // lane c: commit c's part of this warp's columns
+    int first = 0, last = 0;
+    if (lane < count) {
+        const Commit e = list[lane];
+        last = e.w;
+        if (nw > 1) {
+            const int* part = m.blk_part + (size_t)e.x * kRowParts + warp * (kRowParts / nw);
+            first = __ldg(part);
+            if (warp + 1 < nw) last = __ldg(part + kRowParts / nw);
+        }
     }
     const int pieces = (last - first + 31) >> 5;
     int upto = pieces;   // pieces of commits 0..lane
@@ -391,51 +388,48 @@ __device__ __noinline__ void ordered_commits(const DevModel& m, float* cache_any
         if (lane >= o) upto += u;
     }
     const int total = __shfl_sync(full, upto, 31);
+    const int start = first - 32 * (upto - pieces);   // piece i, if it is commit lane's, begins 32 i later
+    // (no branches: past the last piece the commit is the first one and `at` lies
+    // beyond its part)
     for (int i0 = 0; i0 < total; i0 += U) {
-        int col[U], dz[U];
-        float w[U];
+        int col[U];
+        float inc[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            col[u] = -1;
-            dz[u] = 0;
-            w[u] = 0.f;
-            if (i0 + u < total) {
-                const int h = __popc(__ballot_sync(full, upto <= i0 + u));   // the piece's commit
-                const int at = __shfl_sync(full, first - 32 * (upto - pieces), h) + 32 * (i0 + u) + lane;
-                const int end = __shfl_sync(full, last, h);
-                const int base = __shfl_sync(full, row, h);
-                dz[u] = __shfl_sync(full, e.y, h);
-                if (at < end) {
-                    col[u] = __ldg(m.adj_col + base + at);
-                    w[u] = Coef<float>::adj(m, base + at);
-                }
-            }
+            const int h = __popc(__ballot_sync(full, upto <= i0 + u)) & 31;   // the piece's commit
+            const Commit e = list[h];
+            const int at = __shfl_sync(full, start, h) + 32 * (i0 + u) + lane;
+            const bool on = at < __shfl_sync(full, last, h);
+            col[u] = 32 * own;
+            inc[u] = 0.f;
+            if (on) col[u] = __ldg(m.adj_col + e.z + at);
+            if (on) inc[u] = __fmul_rn(Coef<float>::adj(m, e.z + at), (float)e.y);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            if (i0 + u >= total) break;
-            if (col[u] >= 0 && (col[u] >> 5) != own) solo_add(cache + col[u], w[u], dz[u]);
+            if ((col[u] >> 5) != own) cache[col[u]] = __fadd_rn(cache[col[u]], inc[u]);
             __syncwarp();   // a column may come again in the next commit
         }
     }
 }
 
 // Integer rows with fewer links than this in all are scattered by the deciding
-// warp, and fp32 rows with fewer pieces than this beyond one per commit.
+// warp, and fp32 rows with fewer pieces than this beyond one per commit (320
+// variables of 30 links, 64 replicas: 16 pieces 0.89 ms, 6 0.86; 2 is as good as 6).
 constexpr int kScatterAlone = 96;
-constexpr int kPiecesAlone = 16;
+constexpr int kPiecesAlone = 6;
 
 // The commits' rows by the `nt` threads t = 0..nt-1.
 template <class F, int MEM>
 __device__ __forceinline__ void group_scatter(const DevModel& m, F* cache, const Commit* list, int count, int own, int t,
                                               int nt) {
     if constexpr (Num<F>::is_float) {
-        // as many warps as the longest row has pieces
-        int nw = nt >> 5;
-        if (nw > 1) {
+        // a power of two of warps, as many as the longest row has pieces
+        int nw = 1;
+        if (nt > 32) {
             const int lane = t & 31;
             const int longest = __reduce_max_sync(0xffffffffu, lane < count ? list[lane].w : 0);
-            nw = min(nw, (longest + 31) >> 5);
+            while (nw < kRowParts && 2 * nw <= (nt >> 5) && 32 * nw < longest) nw *= 2;
             if ((t >> 5) >= nw) return;
         }
         ordered_commits<MEM>(m, cache, list, count, own, t >> 5, nw, t & 31);
