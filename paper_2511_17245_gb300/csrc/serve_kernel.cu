@@ -124,7 +124,9 @@ __global__ void __launch_bounds__(512, 1) serve_kernel(const ServeArgs s) {
 
 int launch_serve(const ServeArgs& s, int grid, size_t shared_bytes, void* stream) {
     auto kern = dev::serve_kernel;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_bytes);
+    // (one limit for every server: see allow_shared in sweep_launch.cuh)
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         sweep_max_shared_optin() - (int)serve_static_shared());
     if (e != cudaSuccess || grid == 0) return (int)e;
     kern<<<grid, s.rpc * s.tpr, shared_bytes, (cudaStream_t)stream>>>(s);
     return (int)cudaGetLastError();

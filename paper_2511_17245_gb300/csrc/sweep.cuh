@@ -1977,10 +1977,11 @@ constexpr unsigned long long kHandoffSpinLimit = 1ull << 32;
 // it, runs its sweeps and saves the state for the next chunk.  Per-replica
 // results equal those of sweep_kernel: every chunk draws the same Philox
 // counters and the saved state includes the per-thread accumulators.
+using SlicedTasks = int[16][2];
 template <class F, class Z, int RULE, int KIND, bool BLK>
 __global__ void __launch_bounds__(512, 1) sweep_sliced_kernel(const SweepArgs a) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    __shared__ int task_s[16][2];
+    __shared__ SlicedTasks task_s;
     const int slot = threadIdx.x / a.tpr;
     const int t = threadIdx.x - slot * a.tpr;
     if (slot >= a.rpc) return;

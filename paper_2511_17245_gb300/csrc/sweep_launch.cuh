@@ -6,11 +6,20 @@
 
 namespace sa {
 
+// Lets a kernel with `static_bytes` of static shared memory have all the rest as
+// dynamic.  The same limit for every call: one of a call's own size could be
+// lowered by another thread's smaller call before the launch.
+template <class K>
+static cudaError_t allow_shared(K kern, size_t static_bytes = 0) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                sweep_max_shared_optin() - (int)static_bytes);
+}
+
 template <class F, class Z, int RULE, int KIND, bool SMEM, bool BLK>
 static int launch_form(const SweepArgs& a, int blocks, int threads, size_t shared_bytes, cudaStream_t st) {
     auto kern = dev::sweep_kernel<F, Z, RULE, KIND, SMEM, BLK>;
     if (shared_bytes > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_bytes);
+        const cudaError_t e = allow_shared(kern);
         if (e != cudaSuccess) return (int)e;
     }
     kern<<<blocks, threads, shared_bytes, st>>>(a);
@@ -50,7 +59,7 @@ template <class F, class Z, int RULE, int KIND, bool BLK>
 static int launch_sliced_form(const SweepArgs& a, int grid, int threads, size_t shared_bytes, cudaStream_t st,
                               int* blocks_per_sm) {
     auto kern = dev::sweep_sliced_kernel<F, Z, RULE, KIND, BLK>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_bytes);
+    cudaError_t e = allow_shared(kern, sizeof(dev::SlicedTasks));
     if (e != cudaSuccess) return (int)e;
     if (grid == 0) {
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, shared_bytes);
@@ -92,7 +101,7 @@ static int launch_batch_one(const BatchArgs& b, int blocks, int threads, size_t 
                             bool set_attr) {
     auto kern = dev::batch_kernel<F, Z, RULE, KIND, SMEM>;
     if (set_attr) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shared_bytes);
+        const cudaError_t e = allow_shared(kern);
         if (e != cudaSuccess) return (int)e;
     }
     if (blocks == 0) return 0;   // attribute only (before a stream capture)

@@ -141,3 +141,33 @@ def test_a_model_holds_one_record_per_incidence():
     lens = np.diff(inst["term_offsets"])
     incidences = int(lens[lens > 1].sum())
     assert Model(inst).info["device_bytes"] <= 36 * incidences + 200 * 2000 + (1 << 16)
+
+
+def test_calls_of_two_threads_with_different_state_sizes():
+    """Two host threads on streams of their own call the same kernels with 56 and
+    200 KB of shared memory: neither call's limit may reach the other's launch."""
+    import threading
+    errors = []
+
+    def work(n, n_states):
+        try:
+            model = Model(_banded(n, 4000))
+            big = Model(_banded(n_states, 4000))
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                z = torch.ones((1300, n_states), dtype=torch.int32, device="cuda")
+                want = model.run("metropolis", 1, 1, seed=1, threads_per_replica=32)["states"].clone()
+                for _ in range(300):
+                    got = model.run("metropolis", 1, 1, seed=1, threads_per_replica=32)["states"]
+                    big.energy(z)
+                stream.synchronize()
+                assert torch.equal(got, want)
+        except Exception as ex:   # (reported by the main thread)
+            errors.append(ex)
+
+    threads = [threading.Thread(target=work, args=a) for a in ((11_000, 14_000), (40_000, 50_000))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
