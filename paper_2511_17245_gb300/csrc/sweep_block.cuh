@@ -8,7 +8,7 @@
 // lane of the block that shares a term with it changes in the same round, since
 // everything before it in the visiting order is then already in its field; the
 // leading final lanes commit, their changes go into the fields of the other
-// lanes (the 32 x 32 couplings of the block, DevModel::blk_j), and the rest
+// lanes (the 32 x 32 couplings of the block, DevModel::blk_w), and the rest
 // decide again.  The sequential order of Sect. 3.1 is kept exactly, changes are
 // added to a field in that order, and nothing but warp shuffles separates two
 // changes of a block.  Changes reach the other fields block by block.
@@ -442,7 +442,11 @@ __device__ __forceinline__ void group_scatter(const DevModel& m, F* cache, const
 // Block b's couplings, records and masks on their way into one of the two
 // staged places (asynchronous 16-byte copies, issued one block ahead: an
 // L1 prefetch of the same lines left every coupling row an L2 round trip, about
-// 600 cycles a round).
+// 600 cycles a round).  Places lie behind state regions in shared memory alone.
+template <int MEM>
+__device__ __forceinline__ bool blocks_staged(const SweepArgs& a) {
+    return MEM != MEM_GLOBAL && a.off_blk >= 0;
+}
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
@@ -451,7 +455,6 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
-template <int MEM>
 __device__ __forceinline__ void stage_block(const DevModel& m, uint8_t* place, int b, int lane, bool records) {
     const int4* w = reinterpret_cast<const int4*>(m.blk_w + (size_t)b * 1024);
     const int4* rec = reinterpret_cast<const int4*>(m.idx_rec + b * 32);
@@ -459,20 +462,12 @@ __device__ __forceinline__ void stage_block(const DevModel& m, uint8_t* place, i
     int4* dw = reinterpret_cast<int4*>(place);
     int4* dr = reinterpret_cast<int4*>(place + 4096);
     uint32_t* dm = reinterpret_cast<uint32_t*>(place + 4096 + 32 * sizeof(LevelRec));
-    bool shared = MEM == MEM_SHARED;
-    if constexpr (MEM == MEM_EITHER) shared = __isShared(place);
-    if (shared) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) cp_async16(dw + 32 * i + lane, w + 32 * i + lane);
+    for (int i = 0; i < 8; ++i) cp_async16(dw + 32 * i + lane, w + 32 * i + lane);
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-            if (32 * i + lane < 2 * recs) cp_async16(dr + 32 * i + lane, rec + 32 * i + lane);
-        if (lane < recs) cp_async4(dm + lane, m.blk_mask + b * 32 + lane);
-    } else {
-        for (int i = lane; i < 256; i += 32) dw[i] = __ldg(w + i);
-        for (int i = lane; i < 2 * recs; i += 32) dr[i] = __ldg(rec + i);
-        if (lane < recs) dm[lane] = __ldg(m.blk_mask + b * 32 + lane);
-    }
+    for (int i = 0; i < 2; ++i)
+        if (32 * i + lane < 2 * recs) cp_async16(dr + 32 * i + lane, rec + 32 * i + lane);
+    if (lane < recs) cp_async4(dm + lane, m.blk_mask + b * 32 + lane);
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -547,7 +542,7 @@ __device__ __forceinline__ bool sum_in_order(const DevModel& m) {
 
 // Decides block b (warp-collective) from the lanes' fields; on return f holds
 // every change of the block, the list its commits.  Returns their number.
-template <class F, class Z, int RULE>
+template <class F, class Z, int RULE, int MEM>
 __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<F>& q, const uint8_t* place, Z* zs, F& f,
                                             Commit* list, int b, int s, int r, float beta, float temp, int lane,
                                             SweepAcc<F>& acc) {
@@ -555,7 +550,7 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
     const DevModel& m = a.m;
     // row p of the block's couplings
     const int* const blk = reinterpret_cast<const int*>(place) + lane;
-    const bool staged = a.off_blk >= 0;
+    const bool staged = blocks_staged<MEM>(a);
     auto coupling = [&](int p) -> F {
         const size_t at = (size_t)b * 1024 + 32 * p + lane;
         const int w = staged ? blk[32 * p] : __ldg(m.blk_w + at);
@@ -713,7 +708,7 @@ template <class F, class Z, int RULE, int MEM>
 __device__ __forceinline__ void prepare_block(const SweepArgs& a, const Z* zs, uint8_t* place, int b, int s, int r,
                                               int lane, BlockLane<F>& q) {
     if (s >= a.S) return;
-    if (a.off_blk >= 0) stage_block<MEM>(a.m, place, b, lane, false);
+    if (blocks_staged<MEM>(a)) stage_block(a.m, place, b, lane, false);
     q = block_lane<F, Z, RULE>(a, zs, place, false, b, s, r, lane);
 }
 
@@ -741,13 +736,13 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
     // warp 0, at the start of block b: its staged place, with the next block's
     // copies issued (a model of one or two blocks stays staged), and its lanes
     auto begin = [&](int b) -> const uint8_t* {
-        const bool staged = a.off_blk >= 0;
+        const bool staged = blocks_staged<MEM>(a);
         const uint8_t* place = stage + (nb > 2 ? (acc.turn & 1) : b) * kBlockStage;
         if (staged && nb > 2) {
             stage_wait();
             __syncwarp();   // every lane's copies of block b are there; block b - 1's place is free
             ++acc.turn;
-            stage_block<MEM>(m, stage + (acc.turn & 1) * kBlockStage, b + 1 < nb ? b + 1 : 0, lane, true);
+            stage_block(m, stage + (acc.turn & 1) * kBlockStage, b + 1 < nb ? b + 1 : 0, lane, true);
         }
         q = block_lane<F, Z, RULE>(a, zs, place, staged, b, s, r, lane);
         return place;
@@ -782,7 +777,7 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
                     load_rows<F, 1, NR>(ra, m, prev, c, ahead, j);
                     add_rows<F, 1, NR>(ra, f);
                 }
-                const int cnt = decide_block<F, Z, RULE>(a, q, place, zs, f[0], lists + 32 * acc.par, b, s, r, beta,
+                const int cnt = decide_block<F, Z, RULE, MEM>(a, q, place, zs, f[0], lists + 32 * acc.par, b, s, r, beta,
                                                          temp, lane, acc);
                 if (k < m.n) cache[k] = f[0];
                 if (lane == 0) {
@@ -815,7 +810,7 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
                 const int k = b * 32 + lane;
                 F f = k < m.n ? cache[k] : F(0);
                 const uint8_t* place = begin(b);
-                const int cnt = decide_block<F, Z, RULE>(a, q, place, zs, f, lists, b, s, r, beta, temp, lane, acc);
+                const int cnt = decide_block<F, Z, RULE, MEM>(a, q, place, zs, f, lists, b, s, r, beta, temp, lane, acc);
                 if (k < m.n) cache[k] = f;
                 __syncwarp();
                 if (cnt == 0 || nb == 1) continue;
@@ -876,9 +871,9 @@ __device__ __forceinline__ void block_run(const SweepArgs& a, uint8_t* base, int
     if (t < 32) {   // the first block, or all of one or two
         if (a.m.dense_rows && block_pair(tpr, nb)) {
             prepare_block<F, Z, RULE, MEM>(a, zs, stage, 0, s0, r, t, q);
-        } else if (a.off_blk >= 0) {
-            stage_block<MEM>(a.m, stage, 0, t, true);
-            if (nb == 2) stage_block<MEM>(a.m, stage + kBlockStage, 1, t, true);
+        } else if (blocks_staged<MEM>(a)) {
+            stage_block(a.m, stage, 0, t, true);
+            if (nb == 2) stage_block(a.m, stage + kBlockStage, 1, t, true);
             stage_wait();
             __syncwarp();
         }
