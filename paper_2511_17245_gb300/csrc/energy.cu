@@ -356,11 +356,13 @@ template <bool IS_FLOAT, class Z, int G, bool PAIRS>
 int launch_quio_energy(const EnergyArgs& a, cudaStream_t st) {
     auto kern = quio_energy_kernel<IS_FLOAT, Z, G, PAIRS>;
     const size_t sh = (size_t)a.m.n * sizeof(Z) * G;
-    // one limit for every call and size: what a launch may use without it counts
-    // static and dynamic bytes, and a limit of this call's size could be lowered by
-    // another thread's call between here and the launch
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)energy_room());
-    if (e != cudaSuccess) return (int)e;
+    // what a launch may use without a limit of its own, 48 KB, counts static and
+    // dynamic bytes; the limit is the same for every call: one of a call's size could
+    // be lowered by another thread's call before the launch
+    if (sh > 47 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)energy_room());
+        if (e != cudaSuccess) return (int)e;
+    }
     kern<<<(unsigned)((a.n_states + G - 1) / G), 256, sh, st>>>(a);
     return (int)cudaGetLastError();
 }

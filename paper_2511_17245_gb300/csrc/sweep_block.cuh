@@ -70,6 +70,9 @@ __device__ __forceinline__ long long heat_bath_chain(const VarView<F, KIND_QUIO>
     const float zf = __int2float_rn((int)z), v0f = __int2float_rn((int)lo);
     const float b2 = beta * 1.4426950408889634f, mb = Num<F>::to_f(mn) * b2;
     const int n = (int)(c1 - c0) + 1;
+    // the scalar form reaches a value by steps of 1 from its block of 32; beyond
+    // 2^24 the steps round
+    const bool steps_round = Num<F>::is_float && !(fabsf(v0f) + (float)width < 16777216.f);
     float pre[H];
     float sum = 0.f, comp = 0.f;
 #pragma unroll
@@ -80,12 +83,9 @@ __device__ __forceinline__ long long heat_bath_chain(const VarView<F, KIND_QUIO>
             float w = 0.f;
             if (i0 <= c1) {
                 if constexpr (Num<F>::is_float) {
-                    // the value that the scalar form reaches by steps of 1 from
-                    // its block of 32; beyond 2^24 the steps round
-                    const float first = v0f + (float)(c0 + 32u * h);
-                    float vf = first + (float)lane;
-                    if (!(fabsf(first) < 16777216.f - 32.f)) {
-                        vf = first;
+                    float vf = v0f + (float)i0;
+                    if (steps_round) {
+                        vf = v0f + (float)(c0 + 32u * h);
                         for (int i = 0; i < lane; ++i) vf += 1.f;
                     }
                     w = ex2_ftz(fmaf(-vv.delta_ff(zf, vf), b2, mb));
@@ -542,15 +542,16 @@ __device__ __forceinline__ bool sum_in_order(const DevModel& m) {
 
 // Decides block b (warp-collective) from the lanes' fields; on return f holds
 // every change of the block, the list its commits.  Returns their number.
+// `dense` (a constant at each call): a complete graph.
 template <class F, class Z, int RULE, int MEM>
 __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<F>& q, const uint8_t* place, Z* zs, F& f,
                                             Commit* list, int b, int s, int r, float beta, float temp, int lane,
-                                            SweepAcc<F>& acc) {
+                                            SweepAcc<F>& acc, const bool dense) {
     constexpr unsigned full = 0xffffffffu;
     const DevModel& m = a.m;
     // row p of the block's couplings
     const int* const blk = reinterpret_cast<const int*>(place) + lane;
-    const bool staged = blocks_staged<MEM>(a);
+    const bool staged = blocks_staged<MEM>(a), in_order = dense ? Num<F>::is_float : sum_in_order<F>(m);
     auto coupling = [&](int p) -> F {
         const size_t at = (size_t)b * 1024 + 32 * p + lane;
         const int w = staged ? blk[32 * p] : __ldg(m.blk_w + at);
@@ -586,7 +587,7 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
                                                 (wide >> p) & 1u);
             if (vp != zp) {
                 const int dz = vp - zp;
-                if (lane == (sum_in_order<F>(m) ? 0 : p)) {
+                if (in_order ? lane == 0 : lane == p) {
                     const F dp = vv.delta(zp, vp);
                     if constexpr (Num<F>::is_float) acc.de = __fadd_rn(acc.de, (float)dp);   // (no fused multiply-add)
                     else acc.e += dp;
@@ -606,7 +607,6 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
         // A round keeps to one path for all lanes and writes nothing: the list,
         // the state and the energy follow when the block is decided.
         unsigned open = __ballot_sync(full, q.width != 0u), changed = 0u;   // lanes still to be decided, changed
-        const bool chain = m.dense_rows != 0;
         const float u = unit_open_right(q.x.x1);
         // the proposal's share of dE = (v - z) (f + J_kk (v + z)) (quio_delta)
         int dz = 0, dz_done = 0;
@@ -648,7 +648,7 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
             // the first lane whose field one of the changes reaches decides
             // again; on a complete graph that is the next lane
             unsigned done;
-            if (chain) {
+            if (dense) {
                 const unsigned low = c & (0u - c);
                 done = low | (low - 1u);
             } else {
@@ -676,10 +676,10 @@ __device__ __forceinline__ int decide_block(const SweepArgs& a, const BlockLane<
             zs[q.k] = (Z)(v - (long long)q.lo);
             ++acc.changes;
             if constexpr (!Num<F>::is_float) acc.e += de;
-            else if (!sum_in_order<F>(m)) acc.de = __fadd_rn(acc.de, (float)de);
+            else if (!in_order) acc.de = __fadd_rn(acc.de, (float)de);
         }
         if constexpr (Num<F>::is_float) {   // else by one lane, four at a time
-            for (unsigned c = sum_in_order<F>(m) ? changed : 0u; c;) {
+            for (unsigned c = in_order ? changed : 0u; c;) {
                 float ep[4];
                 bool on[4];
 #pragma unroll
@@ -778,7 +778,7 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
                     add_rows<F, 1, NR>(ra, f);
                 }
                 const int cnt = decide_block<F, Z, RULE, MEM>(a, q, place, zs, f[0], lists + 32 * acc.par, b, s, r, beta,
-                                                         temp, lane, acc);
+                                                         temp, lane, acc, true);
                 if (k < m.n) cache[k] = f[0];
                 if (lane == 0) {
                     ctl[acc.par] = cnt;
@@ -810,7 +810,7 @@ __device__ __forceinline__ void block_sweep(const SweepArgs& a, Z* zs, F* cache,
                 const int k = b * 32 + lane;
                 F f = k < m.n ? cache[k] : F(0);
                 const uint8_t* place = begin(b);
-                const int cnt = decide_block<F, Z, RULE, MEM>(a, q, place, zs, f, lists, b, s, r, beta, temp, lane, acc);
+                const int cnt = decide_block<F, Z, RULE, MEM>(a, q, place, zs, f, lists, b, s, r, beta, temp, lane, acc, false);
                 if (k < m.n) cache[k] = f;
                 __syncwarp();
                 if (cnt == 0 || nb == 1) continue;
