@@ -342,7 +342,8 @@ def run_batched_vs_plain(torch, hbm_gbs, sample_every=128, sweep_grid=(250, 500,
     plain_ms, rel_max = plain_time("metropolis", en1000, {i: i for i in everyone})
     plain_total_ms = plain_ms * len(models) / len(sample)
     _progress(f"batched: plain sample {plain_ms:.0f} ms")
-    target = grid[1000]["energy_sum"]   # equal to the plain form's (same seeds; checked on the sample)
+    # the plain form's own (same seeds; their largest difference on the sample is reported)
+    target = grid[1000]["energy_sum"]
     ttt = next(grid[S]["ms"] for S in sweep_grid if grid[S]["energy_sum"] <= target)
     # dense half alone: HBM roofline of its J-row reads
     dense = [i for i in everyone if specs[i]["dense"]]

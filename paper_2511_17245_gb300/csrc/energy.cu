@@ -374,12 +374,15 @@ int launch_quio_form(const EnergyArgs& a, cudaStream_t st) {
     return launch_quio_energy<IS_FLOAT, Z, G, false>(a, st);
 }
 
-// Four states per block when that still gives every SM a few blocks and they
+// Four states per block when that still gives every SM two blocks and they
 // fit, else one; returns false when one state does not fit on chip.
 template <bool IS_FLOAT, class Z>
 bool quio_energy_shape(const EnergyArgs& a, cudaStream_t st, int& rc) {
     const size_t room = energy_room(), one = (size_t)a.m.n * sizeof(Z);
-    if (4 * one <= room && a.n_states >= 4 * 304) rc = launch_quio_form<IS_FLOAT, Z, 4>(a, st);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (4 * one <= room && a.n_states >= 4 * 2 * (int64_t)sms) rc = launch_quio_form<IS_FLOAT, Z, 4>(a, st);
     else if (one <= room) rc = launch_quio_form<IS_FLOAT, Z, 1>(a, st);
     else return false;
     return true;

@@ -286,10 +286,10 @@ inline PlanModel plan_model(const ModelView& v) {
 // A level costs a group barrier, a Philox block and an L2 round trip whatever
 // its width; a block of 32 variables costs one of each plus a short round per
 // colliding change.  kBlockWidth is the mean level width up to which models hold
-// the tables of the blocked sweep (QUIO) and the Metropolis rules use it: 1000
-// variables, 64 replicas x 20 sweeps, blocks against levels 0.66 against 1.96 ms
-// at a width of 7, 2.0 against 4.5 at 13, 2.1 against 5.6 at 15; 1024 replicas
-// 3.4 against 4.8 and 5.8 there.
+// the tables of the blocked sweep (QUIO) and the Metropolis rules use it: 64 /
+// 1024 replicas x 20 sweeps, blocks against the level order, int64, 320 variables
+// of width 7 0.67 / 1.02 against 1.96 / 2.15 ms, 1000 of width 15 2.1 / 3.4 against
+// 5.6 / 5.8; fp32, 1000 of width 13 2.25 / 3.16 against 4.5 / 4.8.
 constexpr int kBlockWidth = 16;
 
 // The heat bath's limit, by the number of values of the widest range.  A block
@@ -339,8 +339,14 @@ constexpr int kBlockStage = 4096 + 32 * (int)sizeof(LevelRec) + 128;
 // several rows deep; else the rows' links).
 inline int plan_blocked_threads(const PlanModel& m) {
     if (m.n <= 32) return 32;
-    // complete graph of 1000 variables, 152 replicas x 50 sweeps: 128 threads
-    // 11.7 ms, 192 7.8, 256 7.0, 384 6.4, 512 7.4
+    // complete fp32 graphs, 152 replicas x 20 sweeps, ms with 64 / 128 / 192 / 256 /
+    // 384 / 512 threads:
+    //    200 variables  0.70   0.62   0.68   0.71   0.72   0.73
+    //    500            3.33   1.76   1.62   1.73   2.13   2.55
+    //   1000           12.8    6.58   4.87   3.97   4.17   5.00
+    //   1998           50.6   25.9   16.3   13.2   14.1   11.4
+    // (600 replicas, four to a block of at most 512 threads: 1000 variables 11.7 ms
+    // with the 128 that fit, 13.7 with 192 and 16.5 with 384)
     if (m.dense_rows) {
         const int want = (m.n * 3 / 8 + 31) / 32 * 32;
         return want > 512 ? 512 : (want < 128 && m.n > 64 ? 128 : want);

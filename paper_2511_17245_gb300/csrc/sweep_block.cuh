@@ -40,7 +40,10 @@ struct SweepAcc {
 // values: one warp issues an instruction every four to five cycles, and the
 // lanes' loops have some 500); in turn, with a variable's values spread over the
 // lanes, it is about 600 a variable.  Above this many changes in the last block
-// they go in turn (the results are the same).
+// they go in turn (the results are the same).  Complete graphs of 32 and 200
+// variables over 4 to 32 values, 64 and 1024 replicas: a limit of 3 costs up to 9%
+// more (6% less for int64 over 4 values, 200 variables), one of 12 from 8% less
+// (fp32) to 11% more (int64, 200 variables, 32 values: 4.72 -> 5.25 ms).
 constexpr int kBusyBlock = 6;
 
 // A change of the block: {variable, z_new - z_old, first entry and length of its row}.
@@ -414,8 +417,10 @@ __device__ __noinline__ void ordered_commits(const DevModel& m, float* cache_any
 }
 
 // Integer rows with fewer links than this in all are scattered by the deciding
-// warp, and fp32 rows with fewer pieces than this beyond one per commit (320
-// variables of 30 links, 64 replicas: 16 pieces 0.89 ms, 6 0.86; 2 is as good as 6).
+// warp (1000 variables of 40 links, 64 replicas x 40 sweeps: 32 links 3.89 ms, 96
+// 3.97, 300 4.36; 320 of 20: 1.19, 1.18, 1.25), and fp32 rows with fewer pieces
+// than this beyond one per commit (320 variables of 30 links, 64 replicas: 16
+// pieces 0.89 ms, 6 0.86; 2 is as good as 6).
 constexpr int kScatterAlone = 96;
 constexpr int kPiecesAlone = 6;
 
