@@ -497,11 +497,12 @@ __device__ __forceinline__ void hb_quio_window(const VarView<F, KIND_QUIO>& vv, 
         vstar = (long long)qv;
     } else {
         vstar = floor_div(-vv.f, 2 * vv.d);
+        if (vstar < lo) vstar = lo;
+        if (vstar > lo + (long long)width) vstar = lo + (long long)width;
     }
-    // (in integers: beyond 2^24 the float of a bound can lie outside of the range)
-    if (vstar < lo) vstar = lo;
-    if (vstar > lo + (long long)width) vstar = lo + (long long)width;
-    const uint32_t bm = (uint32_t)(vstar - lo) / B;
+    // beyond 2^24 the float of a bound can lie outside of the range, and the block
+    // number wrap: the last block then (it is kept only if those before it are)
+    const uint32_t bm = min((uint32_t)(vstar - lo) / B, nblk - 1u);
     if (!kept(bm)) return;  // rounding: keep every block
     uint32_t a = 0, c = bm;  // first kept block in [0, bm]
     while (a < c) { const uint32_t mid = (a + c) / 2; if (kept(mid)) c = mid; else a = mid + 1; }
