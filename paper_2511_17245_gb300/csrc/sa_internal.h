@@ -398,12 +398,12 @@ constexpr int64_t kSlotSlack = 256 * 4;
 // staged blocks of a blocked sweep come after it where they fit, see plan_run.)
 // `zbytes` may exceed the model's own (a batch uses its widest).  QUIO rows are
 // cheap per entry (one atomic) and go inline up to 64 links; HUIO incidences
-// cost a term product each and go inline up to 8.
+// cost a term product each, and every list of them goes to the group.
 inline int64_t plan_layout(const PlanModel& m, int zbytes, int tpr, RunPlan* p) {
     const bool huio = m.kind == KIND_HUIO;
     const int64_t fsize = m.is_float ? 4 : 8;
     p->tpr = tpr;
-    p->heavy_links = huio ? 8 : 64;
+    p->heavy_links = huio ? 0 : 64;
     p->list_cap = huio ? 256 : 64;
     p->off_z = 0;
     p->off_cache = (int32_t)plan_round16((int64_t)m.n * zbytes);

@@ -1734,7 +1734,8 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
         }
     };
     // Applies a decision: state, energy, counters and the neighbours' caches
-    // (inline for short incidence lists, else through the cooperative list).
+    // (QUIO rows up to heavy_links inline, everything else through the cooperative
+    // list while it has places).
     auto apply = [&](const LevelRec& rc, int s, long long z, long long v, F de, int* cnt_now, bool& coop) {
         const int k = rc.k;
         if (v != z) {
@@ -1743,7 +1744,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
             else eacc += (Acc)de;
             ++changes;
             const int len = rc.link_len;
-            // HUIO: every list of incidences is shared by the group (see below)
+            // HUIO: every list of incidences is shared by the group
             bool inline_upd = len <= (KIND == KIND_HUIO ? 0 : a.heavy_links);
             if (!inline_upd) {
                 const int idx = atomicAdd(cnt_now, 1);
@@ -1896,7 +1897,7 @@ __device__ __forceinline__ void replica_body(const SweepArgs& a, const int slot,
             named_bar(bar_id, tpr);
             const int cnt = *cnt_now;
             if (cnt > 0) {
-                // cooperative updates: a hub's list is split over all threads
+                // cooperative updates: the lists are split over all threads
                 const int nl = cnt < a.list_cap ? cnt : a.list_cap;
                 if constexpr (KIND == KIND_HUIO) huio_group_update<F, Z, MEM>(m, zs, cache, list, nl, t, tpr);
                 else quio_group_update<F, MEM>(m, cache, list, nl, t, tpr, solo);
